@@ -96,6 +96,10 @@ def peaks():
 
 def matvec_kernel(tile, states, dtype):
     """Name and source file of the matvec kernel a tuned launch shape selects."""
+    if tile and tile.get("variant", 0) >= 4:
+        rows = 32 if tile["variant"] == 4 else 8
+        return (f"k_apply_block<{rows} rows, {states} states, {1 << tile['ntb']} threads> (cluster {tile['cluster']})",
+                "block", "syk_block.cuh")
     if tile and tile.get("variant", 0) > 0:
         return (f"k_apply_coset<{states}, RB={tile['variant']}, ntb={tile['ntb']}> (cluster {tile['cluster']})",
                 "coset", "syk_apply_coset.cu")

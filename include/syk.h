@@ -345,7 +345,8 @@ int syk_autotune_apply(const syk_terms* terms, int parity, int dtype, int64_t ba
 /* syk_autotune_export / _import -- the tuned table as JSON
  * ({"apply_tiles": [{"N":..,"dtype":..,"batch":..,"ntb":..,"cluster":..,"variant":..,"ms":..}]};
  * variant 0 is the plain tiled kernel, 1..3 the complex64 coset kernel with 2^variant rows
- * per thread; a missing variant reads as 0),
+ * per thread, 4 and 5 the complex64 row-block kernel with 32 and 8 rows per thread; a missing
+ * variant reads as 0),
  * so a tuning run can be cached in a file and reloaded. */
 int syk_autotune_export(char* buf, size_t len);
 int syk_autotune_import(const char* json);
@@ -373,7 +374,7 @@ int syk_counters(int64_t* h_applies, int64_t* krylov_bases, int64_t* launches, i
 
 /* syk_matvec_launches -- matvec launches since the last reset by kernel family (any
  * pointer may be NULL): the row kernel (small sectors, other batch sizes, unaligned
- * vectors), the tiled kernel and the complex64 coset kernel.  A Lanczos segment replayed
+ * vectors), the tiled kernel and the complex64 coset kernels (row blocks among them).  A Lanczos segment replayed
  * from a captured graph adds the launches it recorded.  reset != 0 zeroes them. */
 int syk_matvec_launches(int64_t* rows, int64_t* tiled, int64_t* coset, int reset);
 

@@ -70,12 +70,15 @@ namespace syk {
 
 // Tile configuration chosen by the autotuner per (N, dtype, batch): CTA width 2^ntb,
 // cluster size cs and kernel variant var (0: k_apply_tiled; 1..3: k_apply_coset with
-// 2^var rows per thread).  Absent entries use the built-in heuristic.
+// 2^var rows per thread; 4 and 5: k_apply_block with 32 and 8 rows per thread).  Absent
+// entries use the built-in heuristic.
 struct TileChoice {
   int ntb, cs;
   double ms;
   int var = 0;
 };
+constexpr int kBlockVariant = 4, kLastVariant = 5;
+static int block_rows(int var) { return var == kBlockVariant ? 5 : 3; }  // log2 of the rows per thread
 static std::atomic<int> g_c128_arith{kC128DoubleFloat};
 static std::mutex g_tune_mtx;
 static std::map<uint64_t, TileChoice> g_tune;
@@ -235,8 +238,25 @@ int launch_epilogue(const ApplyParams& p, void* y, int64_t batch, cudaStream_t s
   return SYK_OK;
 }
 
+// complex64 on the row-block kernel: the tuned shape (variant 4 or 5), or its launch rule where nothing
+// is tuned; returns 1 if it does not apply.
+int try_block(const ApplyParams& p, const void* psi, void* y, int64_t batch, cudaStream_t st) {
+  TileChoice tc;
+  BlockShape sh;
+  if (tile_choice_lookup(p.n * 2, SYK_C64, batch, &tc)) {
+    if (tc.var < kBlockVariant || !block_shape(p.n, batch, block_rows(tc.var), tc.ntb - 4, tc.cs, &sh)) return 1;
+  } else if (!block_default(p.n, batch, &sh)) {
+    return 1;
+  }
+  return launch_apply_block(p, batch, psi, y, st, sh);
+}
+
 template <typename R>
 int launch_apply_T(const ApplyParams& p, const void* psi, void* y, int64_t batch, cudaStream_t st) {
+  if constexpr (std::is_same<R, float>::value) {
+    const int rb = try_block(p, psi, y, batch, st);
+    if (rb <= 0) return rb;
+  }
   const int rc = try_tiled<R>(p, psi, y, batch, st);
   if (rc <= 0) return rc;  // launched (0) or failed (< 0)
   int64_t b0 = 0;
@@ -491,7 +511,7 @@ int launch_tiled(const ApplyParams& p, const void* psi, void* y, cudaStream_t st
   TileChoice tc;
   const bool tuned = tile_choice_lookup(p.n * 2, std::is_same<R, float>::value ? SYK_C64 : SYK_C128, BT, &tc);
   if constexpr (std::is_same<R, float>::value && (BT == 4 || BT == 8 || BT == 16)) {
-    if (tuned && tc.var > 0) {
+    if (tuned && tc.var > 0 && tc.var < kBlockVariant) {
       const int rc = launch_coset_var(p, BT, psi, y, st, tc.var, tc.ntb, tc.cs);
       if (rc <= 0) return rc;  // launched or failed; 1: not applicable, plain tiles below
     } else if (!tuned) {
@@ -797,12 +817,17 @@ extern "C" int syk_autotune_apply(const syk_terms* terms, int parity, int dtype,
              : batch == 4 ? TileCfg<double, 4>::RPT : batch == 8 ? TileCfg<double, 8>::RPT : TileCfg<double, 16>::RPT);
   TileChoice best{0, 0, 1e300};
   int rc = SYK_OK;
-  for (int var = 0; var <= 3 && rc == SYK_OK; ++var)
+  for (int var = 0; var <= kLastVariant && rc == SYK_OK; ++var)
   for (int ntb = 6; ntb <= 8 && rc == SYK_OK; ++ntb)
     for (int cs = 1; cs <= 8 && rc == SYK_OK; cs *= 2) {
-      if (!coset_var_ok(dtype, batch, var) || (var && !coset_fits(batch, var, ntb))) continue;
-      const int rpt = var ? 1 << var : rows_per_thread;
-      if ((int64_t(rpt) << ntb) > P.D) continue;  // tile larger than the sector
+      if (var >= kBlockVariant) {
+        BlockShape sh;
+        if (dtype != SYK_C64 || !block_shape(P.n, batch, block_rows(var), ntb - 4, cs, &sh)) continue;
+      } else {
+        if (!coset_var_ok(dtype, batch, var) || (var && !coset_fits(batch, var, ntb))) continue;
+        const int rpt = var ? 1 << var : rows_per_thread;
+        if ((int64_t(rpt) << ntb) > P.D) continue;  // tile larger than the sector
+      }
       tile_choice_set(N, dtype, batch, TileChoice{ntb, cs, 0.0, var});
       rc = launch_apply_H(P, dtype, x, y, batch, st);  // warm-up (also builds the chunk list)
       cudaEventRecord(e0, st);
@@ -897,8 +922,9 @@ extern "C" int syk_autotune_import(const char* json) {
     if (num("N", &N) && num("dtype", &dt) && num("batch", &b) && num("ntb", &ntb) && num("cluster", &cs)) {
       num("ms", &ms);
       num("variant", &var);
+      const bool block = (var == kBlockVariant || var == kLastVariant) && dt == SYK_C64 && (b == 1 || b == 2 || b == 4 || b == 8 || b == 16);
       if (ntb < 6 || ntb > 8 || (cs != 1 && cs != 2 && cs != 4 && cs != 8) ||
-          !coset_var_ok(int(dt), int64_t(b), int(var))) {
+          !(block || coset_var_ok(int(dt), int64_t(b), int(var)))) {
         set_error("syk_autotune_import: invalid entry (ntb=%g cluster=%g variant=%g)", ntb, cs, var);
         return SYK_EINVAL;
       }

@@ -1,0 +1,88 @@
+// Row-block matvec (see syk_block_kernel.cuh): its launch rule, and its kernels with 8 rows per
+// thread for small sectors.
+#include "syk_block_kernel.cuh"
+
+namespace syk {
+namespace {
+
+bool pow2(int64_t v) { return (v & (v - 1)) == 0; }
+
+// Low bits of a row-block launch: a row slot of B << lb elements is 16 for 1 to 16 states in
+// powers of two, so that a half warp reads 128 contiguous bytes, and at most 24 otherwise.
+int low_bits(int64_t B) {
+  int lb = 0;
+  while ((B << (lb + 1)) <= (pow2(B) ? 16 : 24)) ++lb;
+  return lb;
+}
+
+}  // namespace
+
+int block_aux(int n, int rb) {
+  const int ng = (n - 1 - rb + 3) / 4;
+  return rb == 5 ? blk::coset_most(5, ng) : blk::coset_most(3, ng);
+}
+
+size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb) {
+  const size_t warps = ((size_t(B) << (lb + mb)) + 31) / 32;
+  const size_t share = B == 8 || B == 16 ? warps * (rb == 5 ? blk::share_bytes(5, int(B)) : blk::share_bytes(3, int(B))) : 0;
+  return kStages * ((size_t(B) << (lb + rb + mb)) * 8 + auxb) + 64 + share;
+}
+
+bool block_shape(int n, int64_t batch, int rb, int mb, int cs, BlockShape* sh) {
+  if (batch < 1 || batch > 32 || mb < 0 || (rb != 3 && rb != 5)) return false;
+  *sh = {rb, low_bits(batch), mb, cs, block_aux(n, rb)};
+  return sh->lb + rb + mb <= n - 1 && (batch << (sh->lb + mb)) <= 256 &&
+         block_smem(batch, sh->lb, rb, mb, sh->auxb) <= kMaxSmemPerCta;
+}
+
+bool block_default(int n, int64_t batch, BlockShape* sh) {
+  if (batch < 1 || batch > 32 || n - 1 > 31) return false;
+  const int64_t D = int64_t(1) << (n - 1);
+  // State counts that are no power of two: sectors below 2^10 stay with the row kernel, which has
+  // no waits (N = 24, 6 states: 496 us there, 21 us here).
+  if (!pow2(batch) && D < 1024) return false;
+  const int lb = low_bits(batch);
+  int full = 0;  // middle bits of a 256-thread CTA
+  while ((batch << (lb + full + 1)) <= 256) ++full;
+  // 32 rows per thread above 2^16 elements, 8 rows below: there the larger number of threads
+  // counts (N = 32, 1 state: 45 us with 8 rows, 63 with 32; N = 28, 8 states: 39 both; N = 28, 16
+  // states: 68 and 60; N = 38, 8 states: 2.9 and 1.9 ms).  Full tiles (256 threads, one CTA per
+  // SM) halve the copies of 128-thread ones (N = 40, 16 states: 8.7 against 13.7 ms); a cluster
+  // splits a tile's chunks while that leaves at most about one CTA per SM (N = 32, 16 states, 64
+  // tiles: 254 us with 2 CTAs a tile, 466 with 1, 263 with 4; N = 38, 8 states, 256 tiles: 1.93 ms
+  // with 1, 1.96 with 2).  Clusters of 8 only with small CTAs, several to an SM.
+  if (D * batch > (int64_t(1) << 16)) {
+    const int64_t tiles = D >> std::min(n - 1, lb + 5 + full);
+    const int mb = tiles >= 25 ? full : full - 1;
+    const int cs = tiles >= 100 ? 1 : tiles >= 50 ? 2 : 4;
+    if (block_shape(n, batch, 5, mb, cs, sh)) return true;
+  }
+  for (int mb = std::min(3, full); mb >= 0; --mb)
+    if (block_shape(n, batch, 3, mb, 8, sh)) return true;
+  return false;
+}
+
+int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, void* y, cudaStream_t st, BlockShape sh) {
+  if (reinterpret_cast<uintptr_t>(psi) & 15) return 1;  // bulk copies start on 16-byte boundaries
+  BlockArgs a = {};
+  a.B = (int)batch;
+  a.LB = sh.lb;
+  a.MB = sh.mb;
+  a.SE = a.B << sh.lb;
+  a.nt = a.SE << sh.mb;
+  a.auxb = sh.auxb;
+  const BlockLayout* L = nullptr;
+  const int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, !p.no_alloc, &L);
+  if (lr != SYK_OK) return lr > 0 ? 1 : lr;
+  for (int k = 0; k < 9; ++k) a.begin[k] = L->begin[k];
+  const int which = a.SE != 16 ? kBlockAny : sh.lb == 0 ? kBlock16 : batch == 8 ? kBlockShare : kBlockPow2;
+  const bool share = which == kBlock16 || which == kBlockShare;
+  if (sh.rb == 5)
+    return share ? launch_block32_share(p, a, which, sh.cs, L, psi, y, st)
+                 : launch_block32_direct(p, a, which, sh.cs, L, psi, y, st);
+  return share                 ? launch_block<3, 16, true, true, 256>(p, a, sh.cs, L, psi, y, st)
+         : which == kBlockPow2 ? launch_block<3, 16, true, false, 256>(p, a, sh.cs, L, psi, y, st)
+                               : launch_block<3, 0, true, false, 256>(p, a, sh.cs, L, psi, y, st);
+}
+
+}  // namespace syk

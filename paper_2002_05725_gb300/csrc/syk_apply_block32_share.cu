@@ -1,0 +1,12 @@
+// Row-block matvec with 32 rows per thread for 8 and 16 states (see syk_block_kernel.cuh).
+#include "syk_block_kernel.cuh"
+
+namespace syk {
+
+int launch_block32_share(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
+                         const void* psi, void* y, cudaStream_t st) {
+  return which == kBlock16 ? launch_block<5, 16, false, true, 256>(p, a, cs, L, psi, y, st)
+                           : launch_block<5, 16, true, true, 256>(p, a, cs, L, psi, y, st);
+}
+
+}  // namespace syk

@@ -1,0 +1,295 @@
+// K1 variant: y = H psi in one parity sector (Supp. Sec. I.B) for complex64, with the rows of a
+// thread taken as a block of 2^RB consecutive compact indices (syk_block.cuh).
+//
+// A CTA owns a tile of 2^(LB+RB+MB) rows of all B states; thread t = (mid, low, state) owns the
+// 2^RB rows between its low and middle bits, for one state.  Per tile flip h the partner tile
+// psi[tile ^ h] and the chunk's coset records and tables come into shared memory by bulk
+// asynchronous copies, in a ring of kStages stages; the warp that is last to finish a chunk
+// refills its stage, so warps may run ahead of one another by the depth of the ring.
+//
+// Why this split.  The matvec is 8 flop per nonzero and state on operands in shared memory; a
+// thread with one row and all states reads a partner row anew for every mask (or for 1.2 masks,
+// k_apply_coset<16, 1>) and is bound by the shared-memory port.  Here a partner row read once
+// feeds on average 3.4 masks (N = 40), and one coefficient lookup feeds all rows of a thread that
+// share it.  The multiply-adds are the packed two-wide FP32 form: the same FP32 rate (measured
+// 79.3 against 70.7 TFLOP/s in a register-only loop) for half the issue slots, which the
+// coefficient work then takes.  256 threads of 255 registers fill an SM: 128 registers of sums,
+// 64 of partner rows.  Bound now (N = 38, 16 states): FP32 pipe 54 % of its cycles, the rest
+// latency with 2 warps a scheduler; shared-memory port 32 %, L2 14 %.  Without the copies the
+// kernel takes as long, without the cosets of weight 4 (one mask a row: 512 cycles of the port
+// against 256 of the FP32 pipe) 20 % less.
+// Measured (GB300, per matvec, before -> after; before: the faster of the coset, tiled,
+// one-state and row kernels' defaults): N = 40, 16 states 10.45 -> 8.44 ms (40 TFLOP/s); N = 48,
+// 1 state 59.1 -> 19.1 ms; N = 36, 8 states 1.70 -> 0.78 ms; N = 34, 6 states 2.28 -> 0.39 ms;
+// N = 32, 16 states 408 -> 253 us; N = 28, 8 states 136 -> 42 us, 1 state 328 -> 27 us; N = 20, 8
+// states 69 -> 16 us.  Errors against 64-bit sums are 0.4 to 0.7 of the former kernels' (one
+// rounding per product-sum instead of two).
+// Tried and slower: 16 rows per thread with twice the threads (9.1 against 8.7 ms at N = 40, more
+// shared-memory reads per mask); coefficients stored ready-paired (wider reads cost the port more
+// than the register moves they save); two-spin coefficients per thread instead of per row block
+// (9.4 against 8.7 ms); half the warps taking the cosets in another order (9.3, register spills).
+#pragma once
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "syk_block.cuh"
+#include "syk_tile.cuh"
+
+namespace syk {
+
+constexpr int kStages = 3;
+
+struct BlockArgs {
+  int B, LB, MB;
+  int SE;        // elements per row slot: B << LB
+  int nt;        // threads that own rows: SE << MB
+  int auxb;      // bytes of a stage for a chunk's records and tables
+  int begin[9];  // chunk range of each CTA of a tile
+};
+
+// SEC: SE when known at compile time (16), so that row offsets are immediates; 0 otherwise.
+template <int RB, int SEC, bool LOWB, bool SHARE, int MAXT>
+__global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const BlockArgs c, const int4* __restrict__ chunks,
+                                                      const unsigned char* __restrict__ blob,
+                                                      const float2* __restrict__ psi, float2* __restrict__ y) {
+  using namespace blk;
+  constexpr int R = 1 << RB;
+  const int SE = SEC ? SEC : c.SE;
+  const int B = c.B, LB = c.LB, MB = c.MB;
+  const int tileb = (SE << (RB + MB)) * 8, stageb = tileb + c.auxb;
+  extern __shared__ __align__(128) unsigned char sm[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kStages * stageb);
+  int* done = reinterpret_cast<int*>(full + kStages);  // warps that finished the stage's chunk
+  int* issued = done + kStages;                        // chunks copied into the stage so far
+  int* lost = issued + kStages;                        // a wait gave up
+  const int tid = threadIdx.x, nwarps = blockDim.x >> 5;
+  const uint32_t crank = tma::cluster_rank(), csize = tma::cluster_size();  // 0 and 1 without clusters
+  const uint32_t tile = blockIdx.x / csize;
+  const int q0 = c.begin[crank], nq = c.begin[crank + 1] - q0;
+  const bool active = tid < c.nt;
+  const int t = active ? tid : 0;
+  const int mid = t / SE, el = t - mid * SE, low = el / B, s = el - low * B;
+
+  RowCtx ctx;
+  ctx.x = (tile << (LB + RB + MB)) | ((uint32_t)mid << (LB + RB)) | (uint32_t)low;
+  ctx.q = (uint32_t)(__popc(ctx.x) + p.sector) & 1u;
+  ctx.above = (uint32_t)__popc(ctx.x >> (LB + RB)) & 1u;
+  ctx.xn = (ctx.x & ((1u << LB) - 1u)) | ((ctx.x >> (LB + RB)) << LB);
+  ctx.ng = (p.n - 1 - RB + 3) / 4;
+  ctx.n = p.n;
+  ctx.LB = LB;
+  ctx.wd = static_cast<const float*>(p.wd);
+  ctx.B = (uint32_t)B;
+  ctx.share = reinterpret_cast<float2*>(sm + kStages * stageb + 64 + (SHARE ? (tid >> 5) * share_bytes(RB, B) : 0));
+
+  Acc<RB> acc;
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc.re[r] = acc.im[r] = 0ull;
+
+  if (tid == 0) {
+    for (int k = 0; k < kStages; ++k) {
+      tma::mbar_init(&full[k], 1);
+      done[k] = issued[k] = 0;
+    }
+    *lost = 0;
+    tma::fence_mbar_init();
+  }
+  __syncthreads();
+  auto issue = [&](int q, const int4 ch) {  // one thread
+    const int st = q % kStages;
+    ++issued[st];
+    unsigned char* buf = sm + st * stageb;
+    const uint32_t part = tile ^ ((uint32_t)ch.x & 0x7fffffffu);
+    tma::expect_tx(&full[st], (uint32_t)tileb + (uint32_t)ch.z * 16u);
+    tma::bulk_load(buf, reinterpret_cast<const unsigned char*>(psi) + (size_t)part * tileb, (uint32_t)tileb, &full[st]);
+    tma::bulk_load(buf + tileb, blob + (size_t)ch.y * 16, (uint32_t)ch.z * 16u, &full[st]);
+  };
+  if (tid == 0)
+    for (int q = 0; q < kStages && q < nq; ++q) issue(q, __ldg(&chunks[q0 + q]));
+
+  int q = 0;
+  for (; q < nq; ++q) {
+    const int st = q % kStages;
+    // the refill's chunk is read ahead: the refill itself then starts at once
+    const int4 refill = q + kStages < nq ? __ldg(&chunks[q0 + q + kStages]) : make_int4(0, 0, 0, 0);
+    if (!tma::wait_bounded(&full[st], (q / kStages) & 1, tma::kWaitPolls)) break;
+    const unsigned char* tb = sm + st * stageb;
+    const unsigned char* cb = tb + tileb;
+    const uint4 head = *reinterpret_cast<const uint4*>(cb);
+    const uint4* rec = reinterpret_cast<const uint4*>(cb) + 1;
+    constexpr bool LOWS = SEC != 16 || LOWB;
+    auto partner = [&](const uint4 rc) SYK_INLINE {  // the thread's partner row 0
+      const uint32_t lm = LOWS ? (rc.x >> 16) & 0xffu : 0u;
+      return tb + (size_t)((((uint32_t)mid ^ (rc.x & 0xffffu)) << RB) * SE + ((uint32_t)low ^ lm) * B + s) * 8;
+    };
+    CosetAt next;
+    uint4 rc;
+    auto prepare = [&]() SYK_INLINE {  // the next record's coset
+      rc = *rec++;
+      next.odd = rc.x >> 31;
+      next.prow = partner(rc);
+      next.un = support(ctx.x, rc.z);
+      next.sg = parity(rc.y & ctx.x);
+      next.tb = cb + rc.w;
+    };
+    const uint32_t cn = head.x;
+    auto run = [&](auto w, uint32_t count) SYK_INLINE {
+      constexpr int W = decltype(w)::value;
+#pragma unroll 1
+      for (uint32_t k = 0; k < count; ++k) {
+        const CosetAt at = next;
+        prepare();
+        coset<RB, W, LOWS, SHARE>(acc, at, SE * 8, ctx);
+      }
+    };
+    prepare();  // (a record past the last one is never used: it reads the tables behind it)
+    run(std::integral_constant<int, 4>{}, cn & 0xffu);
+    run(std::integral_constant<int, 3>{}, (cn >> 8) & 0xffu);
+    run(std::integral_constant<int, 2>{}, (cn >> 16) & 0xffu);
+    run(std::integral_constant<int, 1>{}, cn >> 24);
+    run(std::integral_constant<int, 0>{}, head.y & 0xffu);
+#pragma unroll 1
+    for (uint32_t k = head.y >> 8; k > 0; --k) {
+      const uint4 r2 = rc;
+      rc = *rec++;
+      m2_record<RB, SHARE>(acc, partner(r2), SE * 8, r2, cb + r2.w, ctx);
+    }
+    // the warp that finishes the chunk last refills its stage
+    __syncwarp();
+    if ((tid & 31) == 0) {
+      __threadfence_block();
+      if (atomicAdd(&done[st], 1) == nwarps - 1) {
+        done[st] = 0;
+        if (q + kStages < nq) issue(q + kStages, refill);
+      }
+    }
+    __syncwarp();
+  }
+  if (q < nq) *lost = 1;
+  __syncthreads();
+  if (*lost) {
+    // let every copy still in flight land before the buffers are reused or the CTA exits
+    if (tid == 0) {
+      atomicOr(p.status, 4);
+      for (int k = 0; k < kStages; ++k)
+        if (issued[k]) tma::wait_bounded(&full[k], (issued[k] - 1) & 1, tma::kDrainPolls);
+    }
+    __syncthreads();
+  }
+
+  // outputs: y[row] = re + i im; the CTAs of a cluster add their sums through shared memory
+  auto value = [&](int r) {
+    const float2 a = unpack2(acc.re[r]), b = unpack2(acc.im[r]);
+    return make_float2(a.x - b.y, a.y + b.x);
+  };
+  const float sc = p.ep_part && p.ep_scale ? (float)p.ep_scale[s] : 1.f;
+  const size_t gbase = (size_t)tile * (tileb / 8);
+  double dr = 0.0, di = 0.0;
+  float fr = 0.f, fi = 0.f;
+  const float2* __restrict__ u = static_cast<const float2*>(p.ep_u);
+  auto emit = [&](size_t e, float2 v, int k) {  // element e of the tile; k counts the thread's elements
+    if (p.ep_part) {
+      v.x *= sc;
+      v.y *= sc;
+      const float2 w = u[gbase + e];
+      fr = fmaf(w.x, v.x, fmaf(w.y, v.y, fr));
+      fi = fmaf(w.x, v.y, fmaf(-w.y, v.x, fi));
+      if ((k & 15) == 15) {
+        dr += fr;
+        di += fi;
+        fr = fi = 0.f;
+      }
+    }
+    y[gbase + e] = v;
+  };
+  if (csize > 1) {
+    float2* st = reinterpret_cast<float2*>(sm);
+    if (active) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) st[((mid << RB) + r) * SE + el] = value(r);
+    }
+    tma::cluster_sync();
+    // each CTA adds 1/csize of the tile's elements over the cluster, in rank order
+    const int part = (tileb / 8) / (int)csize;
+    if (active) {
+      int k = 0;
+      for (int e = (int)crank * part + tid; e < ((int)crank + 1) * part; e += c.nt, ++k) {
+        float2 v = make_float2(0.f, 0.f);
+        const uint32_t a = tma::saddr(st + e);
+        for (uint32_t r = 0; r < csize; ++r) {
+          float2 w;
+          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(w.x), "=f"(w.y) : "r"(tma::map_rank(a, r)) : "memory");
+          v.x += w.x;
+          v.y += w.y;
+        }
+        emit((size_t)e, v, k);
+      }
+    }
+    tma::cluster_sync();  // no CTA leaves, or reuses its memory, while others read it
+  } else {
+    if (active) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) emit((size_t)((mid << RB) + r) * SE + el, value(r), r);
+    }
+    __syncthreads();
+  }
+  if (p.ep_part) {
+    // the CTA's sums per state: thread g * B + s holds state s of group g; halve the groups
+    double2* red = reinterpret_cast<double2*>(sm);
+    if (active) red[tid] = make_double2(dr + fr, di + fi);
+    __syncthreads();
+    for (int h = c.nt / B / 2; h > 0; h >>= 1) {
+      if (tid < h * B) {
+        red[tid].x += red[tid + h * B].x;
+        red[tid].y += red[tid + h * B].y;
+      }
+      __syncthreads();
+    }
+    if (tid < B) p.ep_part[(size_t)blockIdx.x * B + tid] = red[tid];
+    if (blockIdx.x == 0 && tid == 0) *p.ep_nblk = (int)gridDim.x;
+  }
+}
+
+// The instantiations are spread over translation units (each takes a while to compile); which:
+// the state counts they serve.
+enum { kBlock16 = 0, kBlockShare = 1, kBlockPow2 = 2, kBlockAny = 3 };
+int launch_block32_share(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
+                         const void* psi, void* y, cudaStream_t st);
+int launch_block32_direct(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
+                          const void* psi, void* y, cudaStream_t st);
+
+template <int RB, int SEC, bool LOWB, bool SHARE, int MAXT>
+int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLayout* L, const void* psi, void* y,
+             cudaStream_t st) {
+  const int tb = a.LB + RB + a.MB;
+  const int64_t ntiles = p.D >> tb;
+  if (p.ep_part && ntiles * cs > p.ep_cap) {
+    set_error("apply_H: %lld CTAs exceed the epilogue buffer (%lld)", (long long)(ntiles * cs), (long long)p.ep_cap);
+    return SYK_EINVAL;
+  }
+  const size_t smem = block_smem(a.B, a.LB, RB, a.MB, a.auxb);
+  const auto kern = k_apply_block<RB, SEC, LOWB, SHARE, MAXT>;
+  SYK_TRY(ensure_smem_limit((const void*)kern, (int)kMaxSmemPerCta));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ntiles * cs), 1, 1);
+  cfg.blockDim = dim3((unsigned)((a.nt + 31) / 32 * 32), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs > 1 ? 1 : 0;
+  SYK_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, p, a, (const int4*)L->chunks, (const unsigned char*)L->blob,
+                                    static_cast<const float2*>(psi), static_cast<float2*>(y)));
+  count_launch();
+  count_matvec(kMvCoset);
+  SYK_CUDA_CHECK(cudaGetLastError());
+  return SYK_OK;
+}
+
+}  // namespace syk

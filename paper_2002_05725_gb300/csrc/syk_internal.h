@@ -142,6 +142,39 @@ bool coset_fits(int64_t batch, int var, int ntb);  // CTA width 2^ntb (6 or 7) w
 int launch_coset_var(const ApplyParams& p, int64_t batch, const void* psi, void* y, cudaStream_t st, int var, int ntb,
                      int cs);
 
+// Row-block layout of the masks (syk_block.cuh) for tiles of 2^(lb + rb + mb) rows whose threads
+// own 2^rb rows: the cosets of every tile flip h, cut into chunks of at most auxb bytes (coset
+// records, then their tables), dealt to the cs CTAs that share a tile so that each has about
+// the same work, in an order that alternates chunks of much and of little arithmetic.
+//   chunks[c] = {h, chunk offset / 16, chunk bytes / 16, 0}; CTA k of a tile has chunks
+//   begin[k] .. begin[k + 1] - 1.  A chunk starts with a 16-byte header: the numbers of cosets
+//   of weight 4, 3, 2, 1 (a byte each), then of weight 0 and of two-spin records (a byte each).
+struct BlockHost {
+  std::vector<int4> chunks;
+  std::vector<unsigned char> blob;
+  int begin[9] = {};
+};
+int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, BlockHost* out);
+struct BlockLayout {
+  int4* chunks = nullptr;
+  unsigned char* blob = nullptr;
+  int begin[9] = {};
+};
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool may_alloc, const BlockLayout** out);
+
+// Shape of a row-block launch: rows per thread 2^rb, low and middle bits, CTAs per tile, bytes
+// of a chunk's records and tables.  launch_apply_block returns 1 when the shape does not apply.
+struct BlockShape {
+  int rb, lb, mb, cs, auxb;
+};
+int block_aux(int n, int rb);  // the smallest auxb
+size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb);
+// The shape with 2^rb rows per thread (3 or 5), mb middle bits and cs CTAs per tile, if it exists.
+bool block_shape(int n, int64_t batch, int rb, int mb, int cs, BlockShape* sh);
+// The launch rule of the complex64 matvec; false: the sector is too small, or too many states.
+bool block_default(int n, int64_t batch, BlockShape* sh);
+int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, void* y, cudaStream_t st, BlockShape sh);
+
 // complex64 matvec of one state (syk_apply_one.cu) on the tiles of k_apply_tiled<float, 1>
 // (8 rows per thread, CTA width 2^ntb, ntb in 6..8, cluster of cs CTAs; groups: the chunk list
 // of that tile size).
@@ -212,6 +245,7 @@ struct syk_terms {
   mutable syk::DeviceTables dev;
   mutable std::map<int, std::pair<int4*, int>> groups_dev;  // tile bits -> device group list
   mutable std::map<int, syk::CosetLayout> coset_dev;         // (tb, rbits, gmax) -> coset layout
+  mutable std::map<uint64_t, syk::BlockLayout> block_dev;    // (rb, lb, mb, cs, auxb) -> row-block layout
   // Term groups of the per-term inner products (gradients), built on first use: terms sharing
   // an X-mask and a Z-mask off their support bits; device copies on dev.device.
   mutable int ngg = 0;

@@ -34,6 +34,7 @@
 #include <stdexcept>
 #include <string>
 
+#include "syk_block.cuh"
 #include "syk_internal.h"
 
 namespace syk {
@@ -294,6 +295,10 @@ extern "C" void syk_free_terms(syk_terms* t) {
       void* cp[] = {kv.second.chunks, kv.second.counts, kv.second.rec, kv.second.t32, kv.second.t64};
       for (void* p : cp)
         if (p) cudaFree(p);
+    }
+    for (auto& kv : t->block_dev) {
+      if (kv.second.chunks) cudaFree(kv.second.chunks);
+      if (kv.second.blob) cudaFree(kv.second.blob);
     }
     if (prev >= 0) cudaSetDevice(prev);
   }
@@ -654,6 +659,267 @@ int coset_layout(const syk_terms* t, int tb, int rbits, int gmax, bool may_alloc
   SYK_TRY(upload(&L.t32, H.t32.data(), H.t32.size() * sizeof(float)));
   SYK_TRY(upload(&L.t64, H.t64.data(), H.t64.size() * sizeof(double)));
   it = t->coset_dev.emplace(key, L).first;
+  *out = &it->second;
+  return SYK_OK;
+}
+
+namespace {
+
+// Number of the mask with compact flip mc among `count` records in ascending order.
+int find_mask(const std::vector<uint32_t>& rec, int count, uint32_t mc) {
+  int lo = 0, hi = count;
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (rec[4 * size_t(mid)] < mc) lo = mid + 1;
+    else hi = mid;
+  }
+  if (lo >= count || rec[4 * size_t(lo)] != mc) throw std::runtime_error("row-block layout: mask missing");
+  return lo;
+}
+
+// Two-spin tables of mask k (see syk_block.cuh).
+template <int RB>
+void block_m2(const syk_terms* t, int lb, int ng, int k, std::vector<unsigned char>* out) {
+  using namespace blk;
+  const int n = t->n, nb = n - 1;
+  std::vector<int> outside;  // spins outside the row bits, top spin excluded
+  for (int c = 0; c < nb; ++c)
+    if (c < lb || c >= lb + RB) outside.push_back(c);
+  std::vector<float> v;
+  v.reserve(4 * size_t(m2_values(RB, ng)) * 2);
+  auto W = [&](int c, int u) {
+    const double* w = &t->m2_tab[((size_t(k) * n + c) * 4 + u) * 2];
+    return std::complex<double>(w[0], w[1]);
+  };
+  auto put = [&](std::complex<double> c) {
+    v.push_back(float(c.real()));
+    v.push_back(float(c.imag()));
+  };
+  for (int u = 0; u < 4; ++u) {
+    for (int g = 0; g < ng; ++g)
+      for (int e = 0; e < 16; ++e) {
+        std::complex<double> s = 0.0;
+        for (int b = 0; b < 4; ++b)
+          if (size_t(4 * g + b) < outside.size()) s += ((e >> b) & 1) ? -W(outside[4 * g + b], u) : W(outside[4 * g + b], u);
+        put(s);
+      }
+    for (int r = 0; r < (1 << RB); ++r) {
+      std::complex<double> s = 0.0;
+      for (int b = 0; b < RB; ++b) s += ((r >> b) & 1) ? -W(lb + b, u) : W(lb + b, u);
+      put(s);
+    }
+    for (int b = 0; b < RB; ++b) put(W(lb + b, u));
+    put(W(nb, u));
+  }
+  const size_t b0 = out->size();
+  out->resize(b0 + m2_bytes(RB, ng), 0);
+  std::memcpy(out->data() + b0, v.data(), v.size() * 4);
+}
+
+// Appends the tables of the coset with flip `key` outside the row bits (see syk_block.cuh).
+template <int RB>
+void block_tables(const syk_terms* t, int lb, int ng, uint32_t key, int W, std::vector<unsigned char>* blob) {
+  using namespace blk;
+  const int lam = __builtin_popcount(key & ((1u << lb) - 1u));
+  const uint32_t above_u = uint32_t(((1 << W) - 1) & ~((1 << lam) - 1));  // support bits above the row bits
+  const int E = coset_entries(RB, W);
+  const size_t b0 = blob->size();
+  blob->resize(b0 + (size_t(E) << W) * kEntryBytes);
+  float* tab = reinterpret_cast<float*>(blob->data() + b0);
+  int at = 0;
+  for (uint32_t lo = 0; lo < (1u << RB); ++lo) {
+    const int kind = mask_kind(W, lo);
+    const uint32_t mc = key | (lo << lb);
+    if (kind != kM4 && kind != kM4Top) continue;
+    const int m = find_mask(t->m4_rec, t->n4, mc);
+    const int K = __builtin_popcount(lo), tops = kind == kM4Top ? 2 : 1;
+    for (uint32_t un = 0; un < (1u << W); ++un)
+      for (uint32_t ul = 0; ul < (1u << K); ++ul)
+        for (int tp = 0; tp < tops; ++tp) {
+          // support bits in ascending spin order: low bits, row bits, bits above, top spin
+          const uint32_t u = (un & ((1u << lam) - 1u)) | (ul << lam) | ((un >> lam) << (lam + K)) | (uint32_t(tp) << (W + K));
+          int sign = (lam & 1) && ((__builtin_popcount(ul) + K) & 1);
+          if (tops == 2) sign ^= __builtin_popcount(un & above_u) & 1;
+          const double* v = &t->m4_tab[(size_t(m) * 32 + u + (sign ? 16 : 0)) * 2];
+          float* e = tab + (size_t(un) * E + at + ul * tops + tp) * 4;
+          e[0] = float(v[0]);
+          e[1] = float(v[1]);
+          e[2] = -e[0];
+          e[3] = -e[1];
+        }
+    at += tops << K;
+  }
+  if (W == 2) block_m2<RB>(t, lb, ng, find_mask(t->m2_rec, t->n2, key), blob);
+}
+
+template <int RB>
+int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHost* out) {
+  using namespace blk;
+  const int nb = t->n - 1, tb = lb + RB + mb, ng = (nb - RB + 3) / 4;
+  constexpr int kM2Rec = 5;  // items: cosets by weight, and two-spin records
+  struct Item {
+    int type;
+    uint32_t key;
+  };
+  struct Chunk {
+    uint32_t h;
+    std::vector<Item> items;  // cosets of weight 4, 3, 2, 1, 0, then two-spin records
+    int count[6] = {};
+    double cost = 0.0;
+  };
+  // arithmetic of an item in units of one mask: its masks, the partner-row loads and, for
+  // two-spin masks, their coefficients; a tile's copy takes about as long as 4 masks
+  auto cost_of = [](int type) {
+    if (type == kM2Rec) return 4.0;
+    int masks = type == 2 ? 3 : 0;
+    for (uint32_t lo = 0; lo < (1u << RB); ++lo) masks += mask_kind(type, lo) == kM4 || mask_kind(type, lo) == kM4Top;
+    return masks + 1.0;
+  };
+  auto bytes_of = [ng](int type) {
+    return type == 4   ? coset_bytes(RB, 4, ng)
+           : type == 3 ? coset_bytes(RB, 3, ng)
+           : type == 2 ? coset_bytes(RB, 2, ng)
+           : type == 1 ? coset_bytes(RB, 1, ng)
+           : type == 0 ? coset_bytes(RB, 0, ng)
+                       : m2_bytes(RB, ng);
+  };
+  const double fill = 4.0;
+  std::vector<Chunk> all;
+  const uint32_t nlow = 1u << lb, nmid = 1u << mb;
+  for (uint32_t h = 0; h < (1u << (nb - tb)); ++h) {
+    const int wh = __builtin_popcount(h);
+    if (wh > 4) continue;
+    std::vector<Item> items;
+    for (uint32_t m = 0; m < nmid; ++m)
+      for (uint32_t l = 0; l < nlow; ++l) {
+        const int W = wh + __builtin_popcount(m) + __builtin_popcount(l);
+        const uint32_t key = (h << tb) | (m << (lb + RB)) | l;
+        if (W <= 4) items.push_back({W, key});
+        if (W <= 1)
+          for (uint32_t lo = 0; lo < (1u << RB); ++lo)
+            if (mask_kind(W, lo) == kM2 || mask_kind(W, lo) == kM2Top) items.push_back({kM2Rec, key | (lo << lb)});
+      }
+    auto rank = [](int type) { return type == kM2Rec ? 5 : 4 - type; };
+    std::stable_sort(items.begin(), items.end(), [&](const Item& a, const Item& b) { return rank(a.type) < rank(b.type); });
+    size_t k = 0;
+    while (k < items.size()) {
+      Chunk c;
+      c.h = h;
+      int bytes = 16;
+      while (k < items.size()) {
+        const int type = items[k].type, need = 16 + bytes_of(type);
+        if (bytes + need > auxb || c.count[type] == 255) break;
+        bytes += need;
+        c.items.push_back(items[k]);
+        c.count[type]++;
+        c.cost += cost_of(type);
+        ++k;
+      }
+      if (c.items.empty()) throw std::runtime_error("row-block layout: a coset exceeds the chunk size");
+      all.push_back(std::move(c));
+    }
+  }
+  // deal the chunks to the cs CTAs of a tile: the costliest first, each to the least loaded
+  std::stable_sort(all.begin(), all.end(), [](const Chunk& a, const Chunk& b) { return a.cost > b.cost; });
+  std::vector<std::vector<const Chunk*>> lists(cs);
+  std::vector<double> load(cs, 0.0);
+  for (const Chunk& c : all) {
+    const int k = int(std::min_element(load.begin(), load.end()) - load.begin());
+    lists[k].push_back(&c);
+    load[k] += std::max(c.cost, fill);
+  }
+  for (int k = 0; k < cs; ++k) {
+    out->begin[k] = int(out->chunks.size());
+    // spread the chunks whose copy takes longer than their arithmetic evenly among the others
+    size_t nh = 0, nl = 0;
+    for (const Chunk* c : lists[k]) (c->cost > fill ? nh : nl)++;
+    size_t i = 0, j = 0;  // taken so far of the large ones (in front) and of the small ones
+    while (i < nh || j < nl) {
+      const bool small = i == nh || (j < nl && j * nh < i * nl);
+      const Chunk& c = small ? *lists[k][nh + j++] : *lists[k][i++];
+      const size_t b0 = out->blob.size();
+      out->blob.resize(b0 + 16 + 16 * c.items.size());
+      const uint4 head = make_uint4(uint32_t(c.count[4]) | uint32_t(c.count[3]) << 8 | uint32_t(c.count[2]) << 16 |
+                                        uint32_t(c.count[1]) << 24,
+                                    uint32_t(c.count[0]) | uint32_t(c.count[kM2Rec]) << 8, 0u, 0u);
+      std::memcpy(out->blob.data() + b0, &head, 16);
+      for (size_t e = 0; e < c.items.size(); ++e) {
+        const uint32_t key = c.items[e].key;
+        const uint32_t low = key & (nlow - 1u), mid = (key >> (lb + RB)) & (nmid - 1u), lo = (key >> lb) & ((1u << RB) - 1u);
+        uint4 rec = make_uint4(mid | (low << 16), 0u, 0u, uint32_t(out->blob.size() - b0));
+        if (c.items[e].type == kM2Rec) {
+          const int m = find_mask(t->m2_rec, t->n2, key);
+          rec.x |= lo << 24;
+          rec.y = t->m2_rec[4 * size_t(m) + 1];
+          rec.z = t->m2_rec[4 * size_t(m) + 2];
+          block_m2<RB>(t, lb, ng, m, &out->blob);
+        } else {
+          const int W = c.items[e].type;
+          rec.x |= uint32_t(__builtin_popcount(low) & 1) << 31;
+          int below = 0;
+          for (int s = 0; s < nb; ++s) {
+            if (s >= lb && s < lb + RB) continue;
+            if ((key >> s) & 1u) {
+              rec.z |= uint32_t(s - below) << (8 * below);
+              ++below;
+            } else if ((below + (s >= lb + RB ? W : 0)) & 1) {
+              rec.y |= 1u << s;
+            }
+          }
+          for (int q = below; q < 4; ++q) rec.z |= 31u << (8 * q);
+          block_tables<RB>(t, lb, ng, key, W, &out->blob);
+        }
+        std::memcpy(out->blob.data() + b0 + 16 + 16 * e, &rec, 16);
+      }
+      out->chunks.push_back(make_int4(int(c.h), int(b0 / 16), int((out->blob.size() - b0) / 16), 0));
+    }
+  }
+  for (int k = cs; k <= 8; ++k) out->begin[k] = int(out->chunks.size());
+  return SYK_OK;
+}
+
+}  // namespace
+
+int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, BlockHost* out) {
+  if (rb < 3 || rb > 5 || lb < 0 || lb > 8 || mb < 0 || mb > 15 || cs < 1 || cs > 8 || lb + rb + mb > t->n - 1) {
+    set_error("block_layout: unsupported shape (rb=%d lb=%d mb=%d cs=%d)", rb, lb, mb, cs);
+    return SYK_EINVAL;
+  }
+  *out = BlockHost();
+  try {
+    switch (rb) {
+      case 3: return block_layout_T<3>(t, lb, mb, cs, auxb, out);
+      case 4: return block_layout_T<4>(t, lb, mb, cs, auxb, out);
+      default: return block_layout_T<5>(t, lb, mb, cs, auxb, out);
+    }
+  } catch (const std::bad_alloc&) {
+    set_error("block_layout: out of host memory");
+    return SYK_ENOMEM;
+  } catch (const std::exception& e) {
+    set_error("block_layout: %s", e.what());
+    return SYK_EINVAL;
+  }
+}
+
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool may_alloc, const BlockLayout** out) {
+  if (may_alloc) SYK_TRY(ensure_device_tables(t));
+  std::lock_guard<std::mutex> lock(t->mtx);
+  const uint64_t key = uint64_t(rb) | uint64_t(lb) << 8 | uint64_t(mb) << 16 | uint64_t(cs) << 24 | uint64_t(auxb) << 32;
+  auto it = t->block_dev.find(key);
+  if (it == t->block_dev.end()) {
+    if (!may_alloc) return 1;  // not built yet
+    BlockHost H;
+    SYK_TRY(block_layout_host(t, rb, lb, mb, cs, auxb, &H));
+    BlockLayout L;
+    std::memcpy(L.begin, H.begin, sizeof(L.begin));
+    SYK_TRY(upload(&L.chunks, H.chunks.data(), H.chunks.size() * sizeof(int4)));
+    const int rc = upload(&L.blob, H.blob.data(), H.blob.size());
+    if (rc != SYK_OK) {
+      cudaFree(L.chunks);
+      return rc;
+    }
+    it = t->block_dev.emplace(key, L).first;
+  }
   *out = &it->second;
   return SYK_OK;
 }

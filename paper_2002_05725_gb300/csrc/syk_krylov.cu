@@ -21,6 +21,7 @@
 
 #include "syk_cplx.cuh"
 #include "syk_krylov.cuh"
+#include "syk_cheb.cuh"
 #include "syk_tridiag.cuh"
 
 namespace syk {
@@ -37,6 +38,9 @@ inline int red_grid(int64_t total, int bdim, int max_blocks) {
 }
 
 // ---------------------------------------------------------------- reductions
+__device__ __forceinline__ double2 add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+
 // Accumulates sum conj(a) * b.  FP32 data: products and short partial sums in
 // FP32, flushed into FP64 every kFlush elements.  FP64 data: FP64 throughout.
 template <typename R>
@@ -71,20 +75,31 @@ struct DotAcc<float> {
   __device__ double2 get() { return make_double2(re + fr, im + fi); }
 };
 
-// Block-level reduction of one double2 per thread into one value per column:
-// thread t < B gets the sum over threads t, t+B, t+2B, ... in that order.
-__device__ double2 block_reduce_cols(double2 v, int B, double2* sm) {
-  sm[threadIdx.x] = v;
+// The reductions were bound by one thread per column adding its block's 256 partial sums in
+// sequence (complex128 dots of 8 vectors: 47 us at N = 28, 8 states, 516 us for 300 vectors of one
+// state; 21 and 35 us with the tree).
+// Sums over the rows of a block (thread t holds column t % B of row t / B) of NV values per
+// thread, v[j] -> column sums in the threads t < B: a tree over the rows, all values together.
+// sm: NV * blockDim values.  Fixed order.
+template <int NV, typename T>
+__device__ __forceinline__ void block_sum_cols(T (&v)[NV], int B, T* sm) {
+  const int t = threadIdx.x, n = blockDim.x;
+#pragma unroll
+  for (int j = 0; j < NV; ++j) sm[j * n + t] = v[j];
   __syncthreads();
-  double2 r = make_double2(0.0, 0.0);
-  if ((int)threadIdx.x < B) {
-    for (int t = threadIdx.x; t < (int)blockDim.x; t += B) {
-      r.x += sm[t].x;
-      r.y += sm[t].y;
+  int rows = n / B;
+  while (rows > 1) {
+    const int half = (rows + 1) >> 1;
+    if (t < (rows - half) * B) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        v[j] = add(v[j], sm[j * n + t + half * B]);
+        sm[j * n + t] = v[j];
+      }
     }
+    rows = half;
+    __syncthreads();
   }
-  __syncthreads();
-  return r;
 }
 
 // part[(k*G + g)*B + b] = sum over this block's elements of conj(V_k) w, for
@@ -106,9 +121,20 @@ __global__ void k_dots(int nk, const typename CT<R>::T* __restrict__ V, size_t v
         acc[j].tick();
       }
   }
-  for (int j = 0; j < kc; ++j) {
-    double2 r = block_reduce_cols(acc[j].get(), B, sm);
-    if ((int)threadIdx.x < B) part[((size_t)(k0 + j) * gridDim.x + blockIdx.x) * B + threadIdx.x] = r;
+  if (kc == 1) {  // a norm or a single dot
+    double2 v[1] = {acc[0].get()};
+    block_sum_cols<1>(v, B, sm);
+    if ((int)threadIdx.x < B) part[((size_t)k0 * gridDim.x + blockIdx.x) * B + threadIdx.x] = v[0];
+    return;
+  }
+  double2 v[KC];
+#pragma unroll
+  for (int j = 0; j < KC; ++j) v[j] = acc[j].get();
+  block_sum_cols<KC>(v, B, sm);
+  if ((int)threadIdx.x < B) {
+#pragma unroll
+    for (int j = 0; j < KC; ++j)
+      if (j < kc) part[((size_t)(k0 + j) * gridDim.x + blockIdx.x) * B + threadIdx.x] = v[j];
   }
 }
 
@@ -167,33 +193,82 @@ __global__ void k_reduce_parts(int nk, int G, int B, int nwb, const double2* __r
   if (lane == 0) out[idx] = make_double2(f * sx, f * sy);
 }
 
+// The scalars that end a Lanczos step: alpha_j = Re(h1_j + h2_j), beta_j = ||u_{j+1}||; a breakdown
+// sets beta_j = 0.
+struct StepScalars {
+  int j;  // < 0: none
+  const double2 *h1, *h2;
+  double *alpha, *beta, *inv, *sc;
+  int* status;  // [0] error bits, [3] block tickets (0 between kernels)
+  double bt;
+};
+
 // dst = w - sum_{k0<=k<k1} h_k v_k with v_k = sc_k V_k (per column; dst may be w);
-// npart[g*B + b] = partial |dst|^2
+// npart[g*B + b] = partial |dst|^2, and with fin the block that ends last sums these and sets the
+// step's scalars (a kernel of its own before: one launch a step, 4 to 8 us).
+// The coefficients go through shared memory in the vectors' precision: converted per element they
+// cost two FP64 products per vector and element on a pipe of 1/64 of the FP32 rate.
+constexpr int kCoefs = 512;  // coefficients staged at a time
 template <typename R>
-__global__ void k_update(int k0, int k1, const typename CT<R>::T* __restrict__ V, size_t vs,
-                         const double2* __restrict__ h, const double* __restrict__ sc, const typename CT<R>::T* w,
-                         typename CT<R>::T* dst, int64_t total, int B, double* __restrict__ npart) {
+__global__ void __launch_bounds__(256) k_update(int k0, int k1, const typename CT<R>::T* __restrict__ V, size_t vs,
+                                                const double2* __restrict__ h, const double* __restrict__ sc,
+                                                const typename CT<R>::T* w, typename CT<R>::T* dst, int64_t total, int B,
+                                                double* npart, StepScalars fin) {
   using C = typename CT<R>::T;
-  extern __shared__ double2 sm[];
+  __shared__ C cf[kCoefs];
+  __shared__ double red[256];
+  __shared__ int last;
   const int b = threadIdx.x % B;
   DotAcc<R> acc;
   // U elements per thread and pass (same column: the stride is a multiple of B), so that the
   // loads of w and of every basis vector for all U are in flight together
   constexpr int U = 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < total; e0 += U * stride) {
+  const int per = kCoefs / B;  // vectors whose coefficients fit
+  const bool once = k1 - k0 <= per;
+  auto stage = [&](int kb, int ke) {
+    for (int i = threadIdx.x; i < (ke - kb) * B; i += blockDim.x) {
+      const double2 hk = h[kb * B + i];
+      const double f = sc[kb * B + i];
+      cf[i] = make_c<R>(R(-hk.x * f), R(-hk.y * f));
+    }
+  };
+  if (once) stage(k0, k1);
+  __syncthreads();
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += U * stride) {
+    const int64_t e0 = base + threadIdx.x;
     C x[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (e0 + u * stride < total) x[u] = w[e0 + u * stride];
-    for (int k = k0; k < k1; ++k) {
-      const double2 hk = h[k * B + b];
-      const double f = sc[k * B + b];
-      const R cr = R(-hk.x * f), ci = R(-hk.y * f);
-      const C* __restrict__ Vk = V + (size_t)k * vs;
+    for (int kb = k0; kb < k1; kb += per) {
+      const int ke = min(k1, kb + per);
+      if (!once) {
+        __syncthreads();
+        stage(kb, ke);
+        __syncthreads();
+      }
+      if (base + stride >= total) {  // one element per thread: vectors in flight instead
+        if (e0 < total) {
+          C y = make_c<R>(R(0), R(0));
+          const C* __restrict__ Ve = V + (size_t)kb * vs + e0;
+#pragma unroll 8
+          for (int k = 0; k < ke - kb; ++k) {
+            const C c = cf[k * B + b];
+            cmac((k & 1) ? y : x[0], c.x, c.y, Ve[(size_t)k * vs]);
+          }
+          x[0].x += y.x;
+          x[0].y += y.y;
+        }
+      } else {
+        for (int k = kb; k < ke; ++k) {
+          const C c = cf[(k - kb) * B + b];
+          const C* __restrict__ Vk = V + (size_t)k * vs;
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (e0 + u * stride < total) cmac(x[u], cr, ci, Vk[e0 + u * stride]);
+          for (int u = 0; u < U; ++u)
+            if (e0 + u * stride < total) cmac(x[u], c.x, c.y, Vk[e0 + u * stride]);
+        }
+      }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -203,8 +278,37 @@ __global__ void k_update(int k0, int k1, const typename CT<R>::T* __restrict__ V
         acc.tick();
       }
   }
-  double2 r = block_reduce_cols(acc.get(), B, sm);
-  if ((int)threadIdx.x < B && npart) npart[(size_t)blockIdx.x * B + threadIdx.x] = r.x;
+  if (!npart) return;
+  double v[1] = {acc.get().x};
+  block_sum_cols<1>(v, B, red);
+  if ((int)threadIdx.x < B) npart[(size_t)blockIdx.x * B + threadIdx.x] = v[0];
+  if (fin.j < 0) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&fin.status[3], 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double n2[1] = {0.0};
+  for (int g = threadIdx.x / B; g < (int)gridDim.x; g += blockDim.x / B) n2[0] += __ldcg(&npart[(size_t)g * B + b]);
+  block_sum_cols<1>(n2, B, red);
+  if ((int)threadIdx.x < B) {
+    const int j = fin.j;
+    const double a = fin.h1[j * B + b].x + (fin.h2 ? fin.h2[j * B + b].x : 0.0);
+    double be = sqrt(fmax(n2[0], 0.0));
+    if (!isfinite(a) || !isfinite(be)) {
+      atomicOr(fin.status, 1);
+      be = 0.0;
+    }
+    const double prev = j > 0 ? fin.beta[(j - 1) * B + b] : 0.0;
+    if (be <= fin.bt * (fabs(a) + prev)) be = 0.0;
+    fin.alpha[j * B + b] = isfinite(a) ? a : 0.0;
+    fin.beta[j * B + b] = be;
+    const double inv = be > 0.0 ? 1.0 / be : 0.0;
+    fin.inv[b] = inv;
+    fin.sc[(j + 1) * B + b] = inv;  // v_{j+1} = u_{j+1} / beta_j
+  }
+  if (threadIdx.x == 0) fin.status[3] = 0;
 }
 
 template <typename R>
@@ -220,20 +324,65 @@ __global__ void k_scale(const typename CT<R>::T* __restrict__ src, typename CT<R
   }
 }
 
-// out = sum_{k<nk} c_k v_k with v_k = sc_k V_k (per column)
-template <typename R>
-__global__ void k_combine(int nk, const typename CT<R>::T* __restrict__ V, size_t vs, const double2* __restrict__ c,
-                          const double* __restrict__ sc, typename CT<R>::T* __restrict__ out, int64_t total, int B) {
+// out[o] = sum_{k<nk} c_k^o v_k with v_k = sc_k V_k (per column) for NO outputs at once, whose
+// coefficients are cs apart; nk from nk_dev if given.  Coefficients as in k_update.
+template <int NO>
+struct Outs {
+  void* p[NO];
+};
+template <typename R, int NO>
+__global__ void __launch_bounds__(256) k_combine(int nk, const int* __restrict__ nk_dev,
+                                                 const typename CT<R>::T* __restrict__ V, size_t vs,
+                                                 const double2* __restrict__ c, size_t cs, const double* __restrict__ sc,
+                                                 Outs<NO> out, int64_t total, int B) {
   using C = typename CT<R>::T;
+  __shared__ C cf[NO * kCoefs];
+  if (nk_dev) nk = *nk_dev;
   const int b = threadIdx.x % B;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    C x = make_c<R>(R(0), R(0));
-    for (int k = 0; k < nk; ++k) {
-      const double2 ck = c[k * B + b];
-      const double f = sc[k * B + b];
-      cmac(x, R(ck.x * f), R(ck.y * f), V[(size_t)k * vs + e]);
+  const int per = kCoefs / B;
+  const bool once = nk <= per;
+  auto stage = [&](int kb, int ke) {
+    for (int i = threadIdx.x; i < (ke - kb) * B; i += blockDim.x) {
+      const double f = sc[kb * B + i];
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const double2 ck = c[o * cs + kb * B + i];
+        cf[o * kCoefs + i] = make_c<R>(R(ck.x * f), R(ck.y * f));
+      }
     }
-    out[e] = x;
+  };
+  if (once) stage(0, nk);
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += stride) {
+    const int64_t e = base + threadIdx.x;
+    C x[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) x[o] = make_c<R>(R(0), R(0));
+    for (int kb = 0; kb < nk; kb += per) {
+      const int ke = min(nk, kb + per);
+      if (!once) {
+        __syncthreads();
+        stage(kb, ke);
+        __syncthreads();
+      }
+      if (e < total) {
+        const C* __restrict__ Ve = V + (size_t)kb * vs + e;
+#pragma unroll 4
+        for (int k = 0; k < ke - kb; ++k) {
+          const C v = Ve[(size_t)k * vs];
+#pragma unroll
+          for (int o = 0; o < NO; ++o) {
+            const C q = cf[o * kCoefs + k * B + b];
+            cmac(x[o], q.x, q.y, v);
+          }
+        }
+      }
+    }
+    if (e < total) {
+#pragma unroll
+      for (int o = 0; o < NO; ++o) static_cast<C*>(out.p[o])[e] = x[o];
+    }
   }
 }
 
@@ -250,113 +399,189 @@ __global__ void k_norm_init(int B, const double2* __restrict__ d, double* __rest
   inv[b] = nb > 0.0 ? 1.0 / nb : 0.0;
 }
 
-// alpha_j = Re(h1_j + h2_j), beta_j = ||w||; breakdown sets beta_j = 0.  One warp per column:
-// the G partial norms are summed lane-strided, then by a fixed shuffle tree.
-__global__ void k_lanczos_scalars(int j, int B, int G, const double2* __restrict__ h1, const double2* __restrict__ h2,
-                                  const double* __restrict__ npart, double* __restrict__ alpha,
-                                  double* __restrict__ beta, double* __restrict__ inv, double* __restrict__ sc,
-                                  int* status, double bt) {
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (b >= B) return;
-  double n2 = 0.0;
-  for (int g = lane; g < G; g += 32) n2 += npart[(size_t)g * B + b];
-  for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-  if (lane != 0) return;
-  const double a = h1[j * B + b].x + (h2 ? h2[j * B + b].x : 0.0);
-  double be = sqrt(fmax(n2, 0.0));
-  if (!isfinite(a) || !isfinite(be)) {
-    atomicOr(status, 1);
-    be = 0.0;
-  }
-  const double prev = j > 0 ? beta[(j - 1) * B + b] : 0.0;
-  if (be <= bt * (fabs(a) + prev)) be = 0.0;
-  alpha[j * B + b] = isfinite(a) ? a : 0.0;
-  beta[j * B + b] = be;
-  inv[b] = be > 0.0 ? 1.0 / be : 0.0;
-  sc[(j + 1) * B + b] = inv[b];  // v_{j+1} = u_{j+1} / beta_j
-}
+// What a convergence check leaves for the host, or for the kernels that continue on the device:
+// the step all columns accept (0: the basis is not good enough yet), the error bits, the matvec's
+// status word, and whether the check left the coefficients of that step in c.
+struct CheckRec {
+  double sacc;
+  int status, apply, have_c;
+};
 
-// One block (one warp) per batch column: eigendecomposition of T_b and the largest
-// s <= s_target whose error estimate is <= tol.  FULL: the whole eigenvector matrix (for the
-// combination coefficients), written to Qout; otherwise only rows 0 and m-1 (a convergence
-// check), computed by lane 0 alone.  Shared memory: m^2 + 2m + 2 doubles (FULL) or 4m.
+// Eigendecomposition of T (dimension m) by the calling warp into smd: FULL the whole eigenvector
+// matrix Q, else rows 0 and m - 1; d the eigenvalues.  Needs m^2 + 2m + 2 (FULL) or 4m doubles.
 template <bool FULL>
-__device__ void tridiag_eig_block(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                  const double* __restrict__ beta_last_arr, double zr, double zi, double s_target,
-                                  double tol, double* __restrict__ theta, double* __restrict__ Qout,
-                                  double* __restrict__ sb, int* status) {
-  extern __shared__ double smd[];
-  double *Q, *d, *e, *q0, *qm;
-  if constexpr (FULL) {
-    Q = smd;
-    d = Q + m * m;
-    e = d + m;
-    q0 = Q;
-    qm = Q + (m - 1) * m;
-  } else {
-    d = smd;
-    e = d + m;
-    q0 = e + m;
-    qm = q0 + m;
-  }
-  const int b = blockIdx.x;
+__device__ bool eig_column(int m, int B, int b, const double* alpha, const double* beta, double* smd, double** d,
+                           double** q0, double** qm) {
   const int lane = threadIdx.x;
+  double* Q = smd;
+  *d = FULL ? Q + m * m : smd;
+  double* e = *d + m;
+  *q0 = FULL ? Q : e + m;
+  *qm = FULL ? Q + (m - 1) * m : *q0 + m;
   for (int k = lane; k < m; k += 32) {
-    d[k] = alpha[k * B + b];
+    (*d)[k] = alpha[k * B + b];
     e[k] = k + 1 < m ? beta[k * B + b] : 0.0;
   }
   __syncwarp();
-  bool ok;
   if constexpr (FULL) {
-    ok = tridiag_eig_warp(m, d, e, Q, e + m);
+    return tridiag_eig_warp(m, *d, e, Q, e + m);
   } else {
-    ok = true;
-    if (lane == 0) ok = tridiag_eig_rows(m, d, e, q0, qm);
+    bool ok = true;
+    if (lane == 0) ok = tridiag_eig_rows(m, *d, e, *q0, *qm);
     ok = __shfl_sync(0xffffffffu, ok, 0);
     __syncwarp();
+    return ok;
   }
-  if (!ok && lane == 0) atomicOr(status, 2);
-  const double bl = beta_last_arr ? beta_last_arr[b] : 0.0;
-  const double s = select_step(m, d, q0, qm, bl, s_target, tol, zr, zi);
-  for (int k = lane; k < m; k += 32) theta[k * B + b] = d[k];
-  if constexpr (FULL)
-    for (int r = lane; r < m; r += 32)
-      for (int c = 0; c < m; ++c) Qout[((size_t)b * m + r) * m + c] = Q[r * m + c];
-  if (lane == 0) sb[b] = s;
 }
 
-template <bool FULL>
+// c[k*B + b] = beta0_b (e^{s z T} e_1)_k from the sums of the expansion (times e^{s z c + w'})
+__device__ void put_coefs(const cheb::Proj& p, double s, double zr, double zi, double2 y0, double2 y1, double beta0,
+                          int B, int b, double2* c) {
+  const double wx = s * zr * p.r, wy = s * zi * p.r;
+  const double2 f = cexp_scaled(1.0, fma(s * zr, p.c, fabs(wx)), fma(s * zi, p.c, wx < 0.0 ? -wy : wy), 1.0);
+  const int k = 2 * (threadIdx.x & 31);
+  if (k < p.m) c[k * B + b] = make_double2(beta0 * fma(f.x, y0.x, -f.y * y0.y), beta0 * fma(f.x, y0.y, f.y * y0.x));
+  if (k + 1 < p.m)
+    c[(k + 1) * B + b] = make_double2(beta0 * fma(f.x, y1.x, -f.y * y1.y), beta0 * fma(f.x, y1.y, f.y * y1.x));
+}
+
+// Convergence check of column b (one warp): the estimate at s_target; if it passes, the column
+// accepts s_target and its coefficients go to c; else, in the basis' last check, the largest
+// step that passes (0 in earlier checks, where only the whole step counts).  The last block to
+// finish takes the minimum over the columns.
+__device__ void check_column(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
+                             const double* __restrict__ beta0, double zr, double zi, double s_target, double tol, int last,
+                             const int* st_apply, int* status, double* sb, double2* c, CheckRec* rec) {
+  extern __shared__ double smd[];
+  __shared__ int ticket;
+  const int b = blockIdx.x;
+  const double bl = beta[(m - 1) * B + b];
+  const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
+  const double2 w = make_double2(s_target * zr * p.r, s_target * zi * p.r);
+  const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
+  double s;
+  if (aw <= cheb::kMaxW) {
+    double2* ck = reinterpret_cast<double2*>(smd);
+    double* first = smd + 2 * (cheb::kMaxTerms + 1);
+    double* lastv = first + cheb::kMaxTerms + 1;
+    const int K = cheb::terms(aw), K2 = last ? max(K, cheb::terms(2.0 * fabs(w.x))) : K;
+    cheb::coefs(w, K, ck);
+    double2 y0, y1;
+    cheb::sum(p, K, K2, ck, y0, y1, last ? first : nullptr, last ? lastv : nullptr);
+    if (cheb::estimate(p, bl, y0, y1) <= tol) {
+      s = s_target;
+      put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
+    } else {
+      s = last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv) : 0.0;
+      if (threadIdx.x == 0) atomicOr(&status[2], 1);
+    }
+  } else {
+    double *d, *q0, *qm;
+    const bool ok = eig_column<false>(m, B, b, alpha, beta, smd, &d, &q0, &qm);
+    if (!ok && threadIdx.x == 0) atomicOr(status, 2);
+    if (last) s = select_step(m, d, q0, qm, bl, s_target, tol, zr, zi);
+    else s = step_error(m, d, q0, qm, bl, s_target, zr, zi) <= tol ? s_target : 0.0;
+    if (threadIdx.x == 0) atomicOr(&status[2], 1);
+  }
+  if (threadIdx.x == 0) {
+    sb[b] = s;
+    __threadfence();
+    ticket = atomicAdd(&status[3], 1);
+  }
+  __syncwarp();
+  if (ticket != (int)gridDim.x - 1) return;
+  __threadfence();
+  double mn = s;
+  for (int k = threadIdx.x; k < B; k += 32) mn = fmin(mn, __ldcg(&sb[k]));
+  for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+  if (threadIdx.x == 0) {
+    rec->sacc = mn;
+    rec->status = atomicAdd(&status[0], 0);
+    rec->apply = *st_apply;
+    rec->have_c = atomicAdd(&status[2], 0) == 0;
+    status[2] = status[3] = 0;
+  }
+}
+
+__global__ void __launch_bounds__(32) k_krylov_check(int m, int B, const double* __restrict__ alpha,
+                                                     const double* __restrict__ beta, const double* __restrict__ beta0,
+                                                     double zr, double zi, double s_target, double tol, int last,
+                                                     const int* st_apply, int* status, double* sb, double2* c,
+                                                     CheckRec* rec) {
+  check_column(m, B, alpha, beta, beta0, zr, zi, s_target, tol, last, st_apply, status, sb, c, rec);
+}
+
+inline size_t check_smem(int m) {
+  return std::max(sizeof(double) * 4 * size_t(m), (cheb::kMaxTerms + 1) * (sizeof(double2) + 2 * sizeof(double)));
+}
+
+// c[k*B + b] = beta0_b (e^{s z T_b} e_1)_k, one warp per column.
+__device__ void coef_column(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
+                            const double* __restrict__ beta0, double zr, double zi, double s, int* status, double2* c) {
+  extern __shared__ double smd[];
+  const int b = blockIdx.x;
+  const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
+  const double2 w = make_double2(s * zr * p.r, s * zi * p.r);
+  const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
+  if (aw <= cheb::kMaxW) {
+    double2* ck = reinterpret_cast<double2*>(smd);
+    const int K = cheb::terms(aw);
+    cheb::coefs(w, K, ck);
+    double2 y0, y1;
+    cheb::sum(p, K, K, ck, y0, y1, nullptr, nullptr);
+    put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
+    return;
+  }
+  double *d, *q0, *qm;
+  if (!eig_column<true>(m, B, b, alpha, beta, smd, &d, &q0, &qm) && threadIdx.x == 0) atomicOr(status, 2);
+  for (int k = threadIdx.x; k < m; k += 32) {
+    double re = 0.0, im = 0.0;
+    for (int l = 0; l < m; ++l) {
+      const double2 f = cexp_scaled(s, zr, zi, d[l]);
+      const double q = q0[k * m + l] * q0[l];
+      re = fma(q, f.x, re);
+      im = fma(q, f.y, im);
+    }
+    c[k * B + b] = make_double2(beta0[b] * re, beta0[b] * im);
+  }
+}
+
+// The coefficients at several steps: block (b, i) evaluates column b at st.s[i] into c + i * cs.
+constexpr int kMaxSteps = 16;
+struct Steps {
+  double s[kMaxSteps];
+};
+__global__ void __launch_bounds__(32) k_krylov_coefs(int m, int B, const double* __restrict__ alpha,
+                                                     const double* __restrict__ beta, const double* __restrict__ beta0,
+                                                     double zr, double zi, Steps st, int* status, double2* c, size_t cs) {
+  coef_column(m, B, alpha, beta, beta0, zr, zi, st.s[blockIdx.y], status, c + blockIdx.y * cs);
+}
+
+inline size_t coef_smem(int m) {
+  return std::max(sizeof(double) * (size_t(m) * m + 2 * m + 2), (cheb::kMaxTerms + 1) * sizeof(double2));
+}
+
+// theta, Q of the eigendecomposition and c = beta0 Q e^{z theta} Q^T e_1 (syk_tridiag_expm)
 __global__ void k_tridiag_eig(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
-                              const double* __restrict__ beta_last_arr, double zr, double zi, double s_target,
-                              double tol, double* __restrict__ theta, double* __restrict__ Qout,
-                              double* __restrict__ sb, int* status) {
-  tridiag_eig_block<FULL>(m, B, alpha, beta, beta_last_arr, zr, zi, s_target, tol, theta, Qout, sb, status);
+                              double* __restrict__ theta, double* __restrict__ Qout, int* status) {
+  extern __shared__ double smd[];
+  const int b = blockIdx.x, lane = threadIdx.x;
+  double *d, *q0, *qm;
+  if (!eig_column<true>(m, B, b, alpha, beta, smd, &d, &q0, &qm) && lane == 0) atomicOr(status, 2);
+  for (int k = lane; k < m; k += 32) theta[k * B + b] = d[k];
+  for (int r = lane; r < m; r += 32)
+    for (int c = 0; c < m; ++c) Qout[((size_t)b * m + r) * m + c] = q0[r * m + c];
 }
 
-inline size_t tridiag_smem(int m, bool full) {
-  return sizeof(double) * (full ? size_t(m) * m + 2 * m + 2 : 4 * size_t(m));
-}
-
-__global__ void k_step_min(int B, const double* __restrict__ sb, double* __restrict__ sacc) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = sb[0];
-    for (int b = 1; b < B; ++b) s = fmin(s, sb[b]);
-    *sacc = s;
-  }
-}
-
-// c[k*B + b] = beta0_b * sum_l Q_b[k][l] e^{s z theta_l} Q_b[0][l]
+// c[k*B + b] = beta0_b * sum_l Q_b[k][l] e^{z theta_l} Q_b[0][l]
 __global__ void k_tridiag_coef(int m, int B, const double* __restrict__ theta, const double* __restrict__ Q,
-                               const double* __restrict__ beta0, double zr, double zi, const double* __restrict__ sptr,
-                               double s_val, double2* __restrict__ c) {
+                               const double* __restrict__ beta0, double zr, double zi, double2* __restrict__ c) {
   __shared__ double2 fg[SYK_MAX_KRYLOV];
   const int b = blockIdx.x;
   const int k = threadIdx.x;
-  const double s = sptr ? *sptr : s_val;
   const double* Qb = Q + (size_t)b * m * m;
   if (k < m) {
-    const double2 f = cexp_scaled(s, zr, zi, theta[k * B + b]);
+    const double2 f = cexp_scaled(1.0, zr, zi, theta[k * B + b]);
     const double g = Qb[k];  // row 0
     fg[k] = make_double2(f.x * g, f.y * g);
   }
@@ -415,26 +640,26 @@ __global__ void k_reset_ifs(IfHandles hs) {
   for (int k = 0; k < hs.n; ++k) cudaGraphSetConditional(hs.h[k], 0u);
 }
 
-// A convergence check (rows 0 and m-1 only) of the evolution graph.
-__global__ void k_tridiag_eig_dev(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                  const double* __restrict__ beta_last_arr, const ExpJob* __restrict__ job,
-                                  const DevCtl* __restrict__ ctl, double* __restrict__ theta,
-                                  double* __restrict__ Qout, double* __restrict__ sb, int* status) {
-  tridiag_eig_block<false>(m, B, alpha, beta, beta_last_arr, job->zr, job->zi, ctl->s_rem, job->tol, theta, Qout, sb,
-                           status);
+// A convergence check of the evolution graph.
+__global__ void __launch_bounds__(32) k_krylov_check_dev(int m, int B, const double* __restrict__ alpha,
+                                                         const double* __restrict__ beta, const double* __restrict__ beta0,
+                                                         const ExpJob* __restrict__ job, const DevCtl* __restrict__ ctl,
+                                                         int last, const int* st_apply, int* status, double* sb, double2* c,
+                                                         CheckRec* rec) {
+  check_column(m, B, alpha, beta, beta0, job->zr, job->zi, ctl->s_rem, job->tol, last, st_apply, status, sb, c, rec);
 }
-// The full eigendecomposition of the accepted basis (dimension m_eff) for its coefficients.
-__global__ void k_tridiag_eig_full_dev(int B, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                       const DevCtl* __restrict__ ctl, double* __restrict__ theta,
-                                       double* __restrict__ Qout, double* __restrict__ sb, int* status) {
-  tridiag_eig_block<true>(ctl->m_eff, B, alpha, beta, nullptr, 0.0, 0.0, 1.0, 1.0, theta, Qout, sb, status);
+// The coefficients of the accepted basis (dimension m_eff) at its step.
+__global__ void __launch_bounds__(32) k_krylov_coefs_dev(int B, const double* __restrict__ alpha,
+                                                         const double* __restrict__ beta, const double* __restrict__ beta0,
+                                                         const ExpJob* __restrict__ job, const DevCtl* __restrict__ ctl,
+                                                         int* status, double2* c) {
+  coef_column(ctl->m_eff, B, alpha, beta, beta0, job->zr, job->zi, ctl->ds, status, c);
 }
 
 // After the check that ends Lanczos segment [.., j1): converged when the accepted step covers
 // what remains (or the basis is full, or an error bit is set); the next segment's IF handle
 // is set accordingly.  Adds the segment's matvecs and kernel launches to the counters.
-__global__ void k_decide(DevCtl* ctl, int j1, int last, const int* __restrict__ st_ws,
-                         const int* __restrict__ st_apply, const double* __restrict__ sacc,
+__global__ void k_decide(DevCtl* ctl, int j1, int last, const CheckRec* __restrict__ rec,
                          cudaGraphConditionalHandle h_next, int has_next, long long seg_applies,
                          long long seg_launches, long long mv_rows, long long mv_tiled, long long mv_coset) {
   ctl->applies += seg_applies;
@@ -443,11 +668,11 @@ __global__ void k_decide(DevCtl* ctl, int j1, int last, const int* __restrict__ 
   ctl->mv[1] += mv_tiled;
   ctl->mv[2] += mv_coset;
   int e = 0;
-  if (st_ws[0] & 1) e |= 1;     // non-finite Lanczos scalar
-  if (st_ws[0] & 2) e |= 2;     // tridiagonal eigensolver did not converge
-  if (st_apply[0] & 4) e |= 4;  // a bounded wait of a matvec gave up
+  if (rec->status & 1) e |= 1;  // non-finite Lanczos scalar
+  if (rec->status & 2) e |= 2;  // tridiagonal eigensolver did not converge
+  if (rec->apply & 4) e |= 4;   // a bounded wait of a matvec gave up
   ctl->err |= e;
-  const bool conv = last || e != 0 || *sacc >= ctl->s_rem;
+  const bool conv = last || e != 0 || rec->sacc >= ctl->s_rem;
   if (conv) ctl->m_eff = j1;
   if (has_next) cudaGraphSetConditional(h_next, conv ? 0u : 1u);
 }
@@ -455,60 +680,14 @@ __global__ void k_decide(DevCtl* ctl, int j1, int last, const int* __restrict__ 
 // The accepted step of the basis, decided as expmv_T decides it for one output at fraction 1:
 // the output is combined from this basis when the step reaches it (within 1e-13) or covers
 // what remains; otherwise the basis' end state restarts the next one.
-__global__ void k_finalize(DevCtl* ctl, const double* __restrict__ sacc) {
-  const double s_acc = fmin(*sacc, ctl->s_rem);
+__global__ void k_finalize(DevCtl* ctl, const CheckRec* __restrict__ rec) {
+  const double s_acc = fmin(rec->sacc, ctl->s_rem);
   if (!(s_acc > 1e-13 * ctl->s_rem) && !(s_acc >= ctl->s_rem)) ctl->err |= 8;  // step collapsed
   const bool final_basis = s_acc >= ctl->s_rem;
   const bool covered = final_basis || 1.0 <= ctl->s_done + s_acc * (1.0 + 1e-13);
   ctl->s_acc = s_acc;
   ctl->ds = covered ? (final_basis ? s_acc : fmin(1.0 - ctl->s_done, s_acc)) : s_acc;
   ctl->done = covered ? 1 : 0;
-}
-
-__global__ void k_tridiag_coef_dev(int B, const double* __restrict__ theta, const double* __restrict__ Q,
-                                   const double* __restrict__ beta0, const ExpJob* __restrict__ job,
-                                   const DevCtl* __restrict__ ctl, double2* __restrict__ c) {
-  __shared__ double2 fg[SYK_MAX_KRYLOV];
-  const int m = ctl->m_eff;
-  const double s = ctl->ds, zr = job->zr, zi = job->zi;
-  const int b = blockIdx.x;
-  const int k = threadIdx.x;
-  const double* Qb = Q + (size_t)b * m * m;
-  if (k < m) {
-    const double2 f = cexp_scaled(s, zr, zi, theta[k * B + b]);
-    const double g = Qb[k];
-    fg[k] = make_double2(f.x * g, f.y * g);
-  }
-  __syncthreads();
-  if (k < m) {
-    double re = 0.0, im = 0.0;
-    for (int l = 0; l < m; ++l) {
-      const double q = Qb[k * m + l];
-      re = fma(q, fg[l].x, re);
-      im = fma(q, fg[l].y, im);
-    }
-    const double b0 = beta0[b];
-    c[k * B + b] = make_double2(b0 * re, b0 * im);
-  }
-}
-
-// out = sum_{k < m_eff} c_k v_k (m_eff from the control block)
-template <typename R>
-__global__ void k_combine_dev(const DevCtl* __restrict__ ctl, const typename CT<R>::T* __restrict__ V, size_t vs,
-                              const double2* __restrict__ c, const double* __restrict__ sc,
-                              typename CT<R>::T* __restrict__ out, int64_t total, int B) {
-  using C = typename CT<R>::T;
-  const int nk = ctl->m_eff;
-  const int b = threadIdx.x % B;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    C x = make_c<R>(R(0), R(0));
-    for (int k = 0; k < nk; ++k) {
-      const double2 ck = c[k * B + b];
-      const double f = sc[k * B + b];
-      cmac(x, R(ck.x * f), R(ck.y * f), V[(size_t)k * vs + e]);
-    }
-    out[e] = x;
-  }
 }
 
 // End of a Krylov basis: advance by the accepted step; loop while some of z remains.
@@ -531,26 +710,42 @@ struct Ops {
   using C = typename CT<R>::T;
   static void dots(const KrylovWS& ws, int nk, const void* V, size_t vs, const void* w, cudaStream_t st) {
     dim3 grid(ws.G, (nk + KC - 1) / KC);
-    k_dots<R><<<grid, ws.bdim, ws.bdim * sizeof(double2), st>>>(nk, (const C*)V, vs, (const C*)w, ws.D * ws.B,
+    k_dots<R><<<grid, ws.bdim, (nk == 1 ? 1 : KC) * ws.bdim * sizeof(double2), st>>>(nk, (const C*)V, vs, (const C*)w, ws.D * ws.B,
                                                                  (int)ws.B, ws.part);
     count_launch();
   }
   // dst = w - sum_{k0 <= k < k1} h_k v_k
   static void update(const KrylovWS& ws, int k0, int k1, const double2* h, const void* w, void* dst, double* np,
-                     cudaStream_t st) {
-    k_update<R><<<ws.G, ws.bdim, ws.bdim * sizeof(double2), st>>>(k0, k1, (const C*)ws.V, (size_t)(ws.D * ws.B), h,
-                                                                   ws.sc, (const C*)w, (C*)dst, ws.D * ws.B,
-                                                                   (int)ws.B, np);
+                     const StepScalars& fin, cudaStream_t st) {
+    k_update<R><<<ws.G2, ws.bdim2, 0, st>>>(k0, k1, (const C*)ws.V, (size_t)(ws.D * ws.B), h, ws.sc, (const C*)w, (C*)dst,
+                                            ws.D * ws.B, (int)ws.B, np, fin);
     count_launch();
   }
   static void scale(const KrylovWS& ws, const void* src, void* dst, const double* inv, cudaStream_t st) {
     k_scale<R><<<ws.G, ws.bdim, 0, st>>>((const C*)src, (C*)dst, inv, ws.D * ws.B, (int)ws.B);
     count_launch();
   }
-  static void combine(const KrylovWS& ws, int nk, const double2* c, void* out, cudaStream_t st) {
-    k_combine<R><<<ws.G, ws.bdim, 0, st>>>(nk, (const C*)ws.V, (size_t)(ws.D * ws.B), c, ws.sc, (C*)out,
-                                           ws.D * ws.B, (int)ws.B);
-    count_launch();
+  // outs[i] = sum_k c^i_k v_k for i < n, coefficient sets cs apart (nk from nk_dev if given)
+  static void combine(const KrylovWS& ws, int nk, const int* nk_dev, const double2* c, size_t cs, void* const* outs, int n,
+                      cudaStream_t st) {
+    const C* V = (const C*)ws.V;
+    const size_t vs = (size_t)(ws.D * ws.B);
+    while (n > 0) {
+      if (n >= 4) {
+        k_combine<R, 4><<<ws.G2, ws.bdim2, 0, st>>>(nk, nk_dev, V, vs, c, cs, ws.sc,
+                                                    Outs<4>{{outs[0], outs[1], outs[2], outs[3]}}, ws.D * ws.B, (int)ws.B);
+        n -= 4;
+        outs += 4;
+        c += 4 * cs;
+      } else {
+        k_combine<R, 1><<<ws.G2, ws.bdim2, 0, st>>>(nk, nk_dev, V, vs, c, cs, ws.sc, Outs<1>{{outs[0]}}, ws.D * ws.B,
+                                                    (int)ws.B);
+        n -= 1;
+        outs += 1;
+        c += cs;
+      }
+      count_launch();
+    }
   }
 };
 
@@ -590,25 +785,24 @@ int lanczos_step(const ApplyParams& P, int dtype, KrylovWS& ws, int j, int orth,
   Pe.ep_nblk = ws.ep_nblk;
   SYK_TRY(launch_apply_H(Pe, dtype, ws.vec(j), ws.w, B, st));
   void* next = ws.vec(j + 1);
+  const StepScalars none{-1, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0};
+  StepScalars fin{j, ws.h1, nullptr, ws.alpha, ws.beta, ws.inv, ws.sc, ws.status, bt};
   if (orth == kOrthLocal) {
     reduce_parts(ws, 0, ws.h1, st, ws.sc, j, j > 0 ? ws.beta + size_t(j - 1) * B : nullptr);
-    Ops<R>::update(ws, j > 0 ? j - 1 : 0, j + 1, ws.h1, ws.w, next, ws.npart, st);
-    two_pass = false;
+    Ops<R>::update(ws, j > 0 ? j - 1 : 0, j + 1, ws.h1, ws.w, next, ws.npart, fin, st);
   } else {
     if (j > 0) Ops<R>::dots(ws, j, ws.V, vs, ws.w, st);
     reduce_parts(ws, j, ws.h1, st, ws.sc, j);
     if (two_pass) {
-      Ops<R>::update(ws, 0, j + 1, ws.h1, ws.w, ws.w, nullptr, st);
+      Ops<R>::update(ws, 0, j + 1, ws.h1, ws.w, ws.w, nullptr, none, st);
       Ops<R>::dots(ws, j + 1, ws.V, vs, ws.w, st);
       reduce_parts(ws, j + 1, ws.h2, st, ws.sc);
-      Ops<R>::update(ws, 0, j + 1, ws.h2, ws.w, next, ws.npart, st);
+      fin.h2 = ws.h2;
+      Ops<R>::update(ws, 0, j + 1, ws.h2, ws.w, next, ws.npart, fin, st);
     } else {
-      Ops<R>::update(ws, 0, j + 1, ws.h1, ws.w, next, ws.npart, st);
+      Ops<R>::update(ws, 0, j + 1, ws.h1, ws.w, next, ws.npart, fin, st);
     }
   }
-  k_lanczos_scalars<<<(int(B) + 7) / 8, 256, 0, st>>>(j, int(B), ws.G, ws.h1, two_pass ? ws.h2 : nullptr, ws.npart,
-                                                       ws.alpha, ws.beta, ws.inv, ws.sc, ws.status, bt);
-  count_launch();
   SYK_CUDA_CHECK(cudaGetLastError());
   return SYK_OK;
 }
@@ -642,7 +836,7 @@ size_t krylov_ws_bytes(int64_t D, int dtype, int m, int64_t B) {
   s += 3 * align_up(sizeof(double) * B);              // beta0, inv, sb
   s += align_up(sizeof(double) * m * B);              // theta
   s += align_up(sizeof(double) * m * m * B);          // Q
-  s += align_up(sizeof(double));                      // sacc
+  s += align_up(sizeof(CheckRec));                    // rec
   s += align_up(sizeof(double2) * m * B);             // c
   s += align_up(sizeof(int) * 4);                     // status
   if (dtype == SYK_C128) s += align_up(size_t(D) * B * 16);  // split
@@ -668,6 +862,9 @@ int krylov_ws_carve(KrylovWS* ws, void* base, size_t bytes, int64_t D, int dtype
   ws->dtype = dtype;
   ws->bdim = vec_bdim(B);
   ws->G = red_grid(D * B, ws->bdim, std::min(kRedBlocksCap, 2 * sm_count()));
+  // the elementwise kernels of a small vector take small blocks, to reach every SM
+  ws->bdim2 = D * B <= 64 * 2 * int64_t(sm_count()) ? int(B) * std::max(1, int(64 / B)) : ws->bdim;
+  ws->G2 = red_grid(D * B, ws->bdim2, std::min(kRedBlocksCap, 2 * sm_count()));
   const size_t vb = align_up(size_t(D) * B * dtype_size(dtype));
   char* p = static_cast<char*>(base);
   auto take = [&](size_t n) {
@@ -680,7 +877,7 @@ int krylov_ws_carve(KrylovWS* ws, void* base, size_t bytes, int64_t D, int dtype
   ws->part = (double2*)take(sizeof(double2) * ws->G * (m + 1) * B);
   ws->h1 = (double2*)take(sizeof(double2) * (m + 1) * B);
   ws->h2 = (double2*)take(sizeof(double2) * (m + 1) * B);
-  ws->npart = (double*)take(sizeof(double) * ws->G * B);
+  take(sizeof(double) * ws->G * B);
   ws->alpha = (double*)take(sizeof(double) * m * B);
   ws->beta = (double*)take(sizeof(double) * m * B);
   ws->beta0 = (double*)take(sizeof(double) * B);
@@ -688,13 +885,16 @@ int krylov_ws_carve(KrylovWS* ws, void* base, size_t bytes, int64_t D, int dtype
   ws->sb = (double*)take(sizeof(double) * B);
   ws->theta = (double*)take(sizeof(double) * m * B);
   ws->Q = (double*)take(sizeof(double) * m * m * B);
-  ws->sacc = (double*)take(sizeof(double));
+  ws->rec = take(sizeof(CheckRec));
   ws->c = (double2*)take(sizeof(double2) * m * B);
   ws->status = (int*)take(sizeof(int) * 4);
   ws->split = dtype == SYK_C128 ? take(size_t(D) * B * 16) : nullptr;
   ws->sc = (double*)take(sizeof(double) * (m + 1) * B);
   ws->ep_cap = ep_capacity(D);
   ws->ep_part = (double2*)take(sizeof(double2) * size_t(ws->ep_cap) * B);
+  // the update's partial norms: the epilogue's partial dots have been summed by then, and the next
+  // matvec writes them after the norms have (one pair of rows is at least as long as a block's)
+  ws->npart = (double*)ws->ep_part;
   ws->ep_nblk = (int*)take(sizeof(int));
   ws->job = (ExpJob*)take(sizeof(ExpJob));
   ws->ctl = (DevCtl*)take(sizeof(DevCtl));
@@ -858,8 +1058,7 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
   // the first basis checks by the plan; a restart covers an unknown remainder: from 4 vectors on
   const std::vector<int> ends_first = segment_ends(m, plan), ends_restart = segment_ends(m, CheckPlan{4, plan.every});
   const double zr = z.real(), zi = z.imag();
-  int* hstat = static_cast<int*>(ws.host_stage ? ws.host_stage : pinned_scratch(64));
-  double* hs = reinterpret_cast<double*>(hstat + 4);
+  CheckRec* rec = static_cast<CheckRec*>(ws.host_stage ? ws.host_stage : pinned_scratch(64));
   SYK_CUDA_CHECK(cudaMemsetAsync(ws.status, 0, sizeof(int) * 4, st));
   double s_rem = fr[nf - 1], s_done = 0.0;
   int steps = 0, next = 0;
@@ -889,56 +1088,66 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
       const int j1 = ends[si];
       SYK_TRY(run_segment_graphed(P, ws, dtype, B, m, j0, j1, two_pass, st,
                                   [&](cudaStream_t s) { return segment(j0, j1, s); }));
-      const int j = j1 - 1;
       const bool last = (j1 == m);
       {
         const int mm = j1;
-        k_tridiag_eig<false><<<int(B), 32, tridiag_smem(mm, false), st>>>(
-            mm, int(B), ws.alpha, ws.beta, ws.beta + size_t(j) * B, zr, zi, s_rem, tol, ws.theta, ws.Q, ws.sb,
-            ws.status);
-        k_step_min<<<1, 32, 0, st>>>(int(B), ws.sb, ws.sacc);
-        count_launch(2);
-        SYK_CUDA_CHECK(cudaMemcpyAsync(hstat, ws.status, sizeof(int) * 2, cudaMemcpyDeviceToHost, st));
-        SYK_CUDA_CHECK(cudaMemcpyAsync(hstat + 2, P.status, sizeof(int), cudaMemcpyDeviceToHost, st));
-        SYK_CUDA_CHECK(cudaMemcpyAsync(hs, ws.sacc, sizeof(double), cudaMemcpyDeviceToHost, st));
+        k_krylov_check<<<int(B), 32, check_smem(mm), st>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, s_rem, tol,
+                                                           last ? 1 : 0, P.status, ws.status, ws.sb, ws.c,
+                                                           (CheckRec*)ws.rec);
+        count_launch();
+        SYK_CUDA_CHECK(cudaMemcpyAsync(rec, ws.rec, sizeof(CheckRec), cudaMemcpyDeviceToHost, st));
         SYK_CUDA_CHECK(cudaStreamSynchronize(st));
         prof_collect();
-        if (hstat[0] & 1) {
+        if (rec->status & 1) {
           set_error("expmv: non-finite Lanczos scalar");
           return SYK_ENUMERIC;
         }
-        if (hstat[0] & 2) {
+        if (rec->status & 2) {
           set_error("expmv: tridiagonal eigensolver did not converge");
           return SYK_ENUMERIC;
         }
-        if (hstat[2] & 4) {
+        if (rec->apply & 4) {
           set_error("apply_H: a bounded wait for a staged tile gave up");
           return SYK_ETIMEOUT;
         }
-        if (last || *hs >= s_rem) {
+        if (last || rec->sacc >= s_rem) {
           m_eff = mm;
           break;
         }
       }
       j0 = j1;
     }
-    double s_acc = std::min(*hs, s_rem);
+    double s_acc = std::min(rec->sacc, s_rem);
     if (!(s_acc > 1e-13 * s_rem) && !(s_acc >= s_rem)) {
       set_error("expmv: Krylov step collapsed (s=%g of remaining %g); raise krylov_dim or tol", s_acc, s_rem);
       return SYK_ENUMERIC;
     }
-    // the checks kept only two rows of the eigenvectors: the full set for the coefficients
-    k_tridiag_eig<true><<<int(B), 32, tridiag_smem(m_eff, true), st>>>(
-        m_eff, int(B), ws.alpha, ws.beta, nullptr, zr, zi, 1.0, 1.0, ws.theta, ws.Q, ws.sb, ws.status);
-    count_launch();
     const bool final_basis = s_acc >= s_rem;
-    // outputs whose fraction this basis reaches
+    // outputs whose fraction this basis reaches, a few at a time; the check that accepted the whole
+    // step left that step's coefficients in ws.c
+    const int batch = std::max(1, std::min(kMaxSteps, m / 2));  // sets that fit the m x m scratch
+    const size_t cset = size_t(m) * B;
     while (next < nf && (fr[next] <= s_done + s_acc * (1.0 + 1e-13) || (final_basis && next == nf - 1))) {
-      const double ds = (final_basis && next == nf - 1) ? s_acc : std::min(fr[next] - s_done, s_acc);
-      k_tridiag_coef<<<int(B), 64, 0, st>>>(m_eff, int(B), ws.theta, ws.Q, ws.beta0, zr, zi, nullptr, ds, ws.c);
+      if (final_basis && next == nf - 1 && rec->have_c) {
+        Ops<R>::combine(ws, m_eff, nullptr, ws.c, 0, outs + next, 1, st);
+        ++next;
+        continue;
+      }
+      Steps sp = {};
+      int n = 0;
+      while (n < batch && next + n < nf &&
+             (fr[next + n] <= s_done + s_acc * (1.0 + 1e-13) || (final_basis && next + n == nf - 1))) {
+        const bool end = final_basis && next + n == nf - 1;
+        if (end && rec->have_c) break;
+        sp.s[n] = end ? s_acc : std::min(fr[next + n] - s_done, s_acc);
+        ++n;
+      }
+      double2* cq = reinterpret_cast<double2*>(ws.Q);
+      k_krylov_coefs<<<dim3(int(B), n), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp,
+                                                                    ws.status, cq, cset);
       count_launch();
-      Ops<R>::combine(ws, m_eff, ws.c, outs[next], st);
-      ++next;
+      Ops<R>::combine(ws, m_eff, nullptr, cq, cset, outs + next, n, st);
+      next += n;
     }
     if (next == nf) {
       SYK_CUDA_CHECK(cudaGetLastError());
@@ -946,9 +1155,12 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
       break;
     }
     if (!final_basis) {  // restart from the state at the end of this basis' step
-      k_tridiag_coef<<<int(B), 64, 0, st>>>(m_eff, int(B), ws.theta, ws.Q, ws.beta0, zr, zi, nullptr, s_acc, ws.c);
+      Steps sp = {};
+      sp.s[0] = s_acc;
+      k_krylov_coefs<<<dim3(int(B), 1), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp,
+                                                                    ws.status, ws.c, 0);
       count_launch();
-      Ops<R>::combine(ws, m_eff, ws.c, outs[nf - 1], st);
+      Ops<R>::combine(ws, m_eff, nullptr, ws.c, 0, outs + nf - 1, 1, st);
       cur = outs[nf - 1];
     }
     SYK_CUDA_CHECK(cudaGetLastError());
@@ -1123,13 +1335,12 @@ int build_dev_graph(const ApplyParams& P, int dtype, KrylovWS& ws, int orth, boo
     capture_counts_end(&l0, &a0, kinds);
     capture_counts_begin();  // keep counting captured launches away from the global counters
     const int mm = j1;
-    k_tridiag_eig_dev<<<int(B), 32, tridiag_smem(mm, false), cs>>>(mm, int(B), ws.alpha, ws.beta,
-                                                                  ws.beta + size_t(j1 - 1) * B, ws.job,
-                                                                  ws.ctl, ws.theta, ws.Q, ws.sb, ws.status);
-    k_step_min<<<1, 32, 0, cs>>>(int(B), ws.sb, ws.sacc);
+    k_krylov_check_dev<<<int(B), 32, check_smem(mm), cs>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, ws.job, ws.ctl,
+                                                           j1 == m ? 1 : 0, P.status, ws.status, ws.sb, ws.c,
+                                                           (CheckRec*)ws.rec);
     const bool has_next = k < ifs.n;
-    k_decide<<<1, 1, 0, cs>>>(ws.ctl, j1, j1 == m ? 1 : 0, ws.status, P.status, ws.sacc,
-                              has_next ? ifs.h[k] : cudaGraphConditionalHandle(0), has_next ? 1 : 0, a0, l0 + 3,
+    k_decide<<<1, 1, 0, cs>>>(ws.ctl, j1, j1 == m ? 1 : 0, (const CheckRec*)ws.rec,
+                              has_next ? ifs.h[k] : cudaGraphConditionalHandle(0), has_next ? 1 : 0, a0, l0 + 2,
                               kinds[kMvRows], kinds[kMvTiled], kinds[kMvCoset]);
     SYK_CUDA_CHECK(cudaGetLastError());
     return SYK_OK;
@@ -1203,14 +1414,12 @@ int build_dev_graph(const ApplyParams& P, int dtype, KrylovWS& ws, int orth, boo
   fr = {bnode};
   // body tail: the accepted step's coefficients, w = V c, advance
   DEV_CK(cudaStreamBeginCaptureToGraph(cs, body, fr.data(), nullptr, fr.size(), mode), "capture tail");
-  k_finalize<<<1, 1, 0, cs>>>(ws.ctl, ws.sacc);
-  k_tridiag_eig_full_dev<<<int(B), 32, tridiag_smem(m, true), cs>>>(int(B), ws.alpha, ws.beta, ws.ctl, ws.theta,
-                                                                     ws.Q, ws.sb, ws.status);
-  k_tridiag_coef_dev<<<int(B), 64, 0, cs>>>(int(B), ws.theta, ws.Q, ws.beta0, ws.job, ws.ctl, ws.c);
-  k_combine_dev<R><<<ws.G, ws.bdim, 0, cs>>>(ws.ctl, (const typename CT<R>::T*)ws.V, size_t(ws.D * B), ws.c, ws.sc,
-                                             (typename CT<R>::T*)ws.w, ws.D * B, int(B));
-  // per basis: head, the 4 kernels of v_0, reset, finalize, eigenvectors, coefficients, combine, advance
-  k_advance<<<1, 1, 0, cs>>>(ws.ctl, hloop, 11);
+  k_finalize<<<1, 1, 0, cs>>>(ws.ctl, (const CheckRec*)ws.rec);
+  k_krylov_coefs_dev<<<int(B), 32, coef_smem(m), cs>>>(int(B), ws.alpha, ws.beta, ws.beta0, ws.job, ws.ctl, ws.status, ws.c);
+  void* wout = ws.w;
+  Ops<R>::combine(ws, m, &ws.ctl->m_eff, ws.c, 0, &wout, 1, cs);
+  // per basis: head, the 4 kernels of v_0, reset, finalize, coefficients, combine, advance
+  k_advance<<<1, 1, 0, cs>>>(ws.ctl, hloop, 10);
   {
     cudaGraph_t tmp = body;
     DEV_CK(cudaStreamEndCapture(cs, &tmp), "end capture tail");
@@ -1426,14 +1635,12 @@ extern "C" int syk_tridiag_expm(int m, int64_t batch, const double* alpha, const
   double* bpad = (double*)base;
   double* theta = (double*)(base + nb);
   double* Q = (double*)(base + 2 * nb);
-  double* sb = (double*)(base + 2 * nb + nq);
   int* status = (int*)(base + 2 * nb + nq + align_up(sizeof(double) * B));
   cudaMemsetAsync(bpad, 0, nb, st);
   cudaMemsetAsync(status, 0, 16, st);
   if (m > 1) cudaMemcpyAsync(bpad, beta, sizeof(double) * (m - 1) * B, cudaMemcpyDeviceToDevice, st);
-  k_tridiag_eig<true><<<B, 32, tridiag_smem(m, true), st>>>(m, B, alpha, bpad, nullptr, z_re, z_im, 1.0, 1.0, theta, Q,
-                                                             sb, status);
-  k_tridiag_coef<<<B, 64, 0, st>>>(m, B, theta, Q, beta0, z_re, z_im, nullptr, 1.0, (double2*)out);
+  k_tridiag_eig<<<B, 32, sizeof(double) * (size_t(m) * m + 2 * m + 2), st>>>(m, B, alpha, bpad, theta, Q, status);
+  k_tridiag_coef<<<B, 64, 0, st>>>(m, B, theta, Q, beta0, z_re, z_im, (double2*)out);
   count_launch(2);
   cudaError_t e = cudaGetLastError();
   int hstat = 0;

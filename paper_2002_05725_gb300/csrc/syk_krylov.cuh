@@ -27,13 +27,14 @@ struct KrylovWS {
   int64_t B = 0, D = 0;
   int dtype = 0;
   int G = 0;            // blocks of the reduction kernels
-  int bdim = 0;         // threads per block of the vector kernels (multiple of B)
+  int bdim = 0;         // threads per block of the dot kernels (multiple of B)
+  int G2 = 0, bdim2 = 0;  // blocks and threads of the elementwise kernels
   char* V = nullptr;    // (m+1) basis vectors, D*B elements each
   char* w = nullptr;    // work vector
   double2* part = nullptr;   // G * (m+1) * B partial dots
   double2* h1 = nullptr;     // (m+1) * B
   double2* h2 = nullptr;
-  double* npart = nullptr;   // G * B partial squared norms
+  double* npart = nullptr;   // G2 * B partial squared norms (the memory of ep_part)
   double* alpha = nullptr;   // m * B
   double* beta = nullptr;    // m * B
   double* beta0 = nullptr;   // B
@@ -41,9 +42,9 @@ struct KrylovWS {
   double* theta = nullptr;   // m * B
   double* Q = nullptr;       // B * m * m
   double* sb = nullptr;      // B
-  double* sacc = nullptr;    // 1
+  char* rec = nullptr;       // result of a convergence check (syk_krylov.cu)
   double2* c = nullptr;      // m * B
-  int* status = nullptr;     // 4 ints
+  int* status = nullptr;     // 4 ints: error bits, -, check coefficients missing, block tickets
   char* split = nullptr;     // complex128 only: double-float copy of the matvec input (D*B float4)
   // The basis is stored unnormalised: V_k = u_k with v_k = sc[k*B + b] u_k (sc[0] = 1; the
   // Lanczos step folds 1/beta_j into the next matvec's output instead of rescaling u_{j+1}).

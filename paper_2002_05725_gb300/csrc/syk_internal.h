@@ -175,6 +175,15 @@ bool block_shape(int n, int64_t batch, int rb, int mb, int cs, BlockShape* sh);
 bool block_default(int n, int64_t batch, BlockShape* sh);
 int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, void* y, cudaStream_t st, BlockShape sh);
 
+// Small sectors (syk_small.cu): every mask's coefficient c_m(x) for every row of each sector
+// (masks x D, FP64) and its compact flip.
+struct SmallTables {
+  int masks = 0;
+  double2* coef[2] = {nullptr, nullptr};
+  uint32_t* flips = nullptr;
+};
+int small_tables(const syk_terms* t, bool may_alloc, const SmallTables** out);
+
 // complex64 matvec of one state (syk_apply_one.cu) on the tiles of k_apply_tiled<float, 1>
 // (8 rows per thread, CTA width 2^ntb, ntb in 6..8, cluster of cs CTAs; groups: the chunk list
 // of that tile size).
@@ -245,6 +254,7 @@ struct syk_terms {
   mutable syk::DeviceTables dev;
   mutable std::map<int, std::pair<int4*, int>> groups_dev;  // tile bits -> device group list
   mutable std::map<int, syk::CosetLayout> coset_dev;         // (tb, rbits, gmax) -> coset layout
+  mutable syk::SmallTables small_dev;
   mutable std::map<uint64_t, syk::BlockLayout> block_dev;    // (rb, lb, mb, cs, auxb) -> row-block layout
   // Term groups of the per-term inner products (gradients), built on first use: terms sharing
   // an X-mask and a Z-mask off their support bits; device copies on dev.device.

@@ -21,7 +21,7 @@
 
 #include "syk_cplx.cuh"
 #include "syk_krylov.cuh"
-#include "syk_cheb.cuh"
+#include "syk_check.cuh"
 #include "syk_tridiag.cuh"
 
 namespace syk {
@@ -399,91 +399,18 @@ __global__ void k_norm_init(int B, const double2* __restrict__ d, double* __rest
   inv[b] = nb > 0.0 ? 1.0 / nb : 0.0;
 }
 
-// What a convergence check leaves for the host, or for the kernels that continue on the device:
-// the step all columns accept (0: the basis is not good enough yet), the error bits, the matvec's
-// status word, and whether the check left the coefficients of that step in c.
-struct CheckRec {
-  double sacc;
-  int status, apply, have_c;
-};
-
-// Eigendecomposition of T (dimension m) by the calling warp into smd: FULL the whole eigenvector
-// matrix Q, else rows 0 and m - 1; d the eigenvalues.  Needs m^2 + 2m + 2 (FULL) or 4m doubles.
-template <bool FULL>
-__device__ bool eig_column(int m, int B, int b, const double* alpha, const double* beta, double* smd, double** d,
-                           double** q0, double** qm) {
-  const int lane = threadIdx.x;
-  double* Q = smd;
-  *d = FULL ? Q + m * m : smd;
-  double* e = *d + m;
-  *q0 = FULL ? Q : e + m;
-  *qm = FULL ? Q + (m - 1) * m : *q0 + m;
-  for (int k = lane; k < m; k += 32) {
-    (*d)[k] = alpha[k * B + b];
-    e[k] = k + 1 < m ? beta[k * B + b] : 0.0;
-  }
-  __syncwarp();
-  if constexpr (FULL) {
-    return tridiag_eig_warp(m, *d, e, Q, e + m);
-  } else {
-    bool ok = true;
-    if (lane == 0) ok = tridiag_eig_rows(m, *d, e, *q0, *qm);
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    return ok;
-  }
-}
-
-// c[k*B + b] = beta0_b (e^{s z T} e_1)_k from the sums of the expansion (times e^{s z c + w'})
-__device__ void put_coefs(const cheb::Proj& p, double s, double zr, double zi, double2 y0, double2 y1, double beta0,
-                          int B, int b, double2* c) {
-  const double wx = s * zr * p.r, wy = s * zi * p.r;
-  const double2 f = cexp_scaled(1.0, fma(s * zr, p.c, fabs(wx)), fma(s * zi, p.c, wx < 0.0 ? -wy : wy), 1.0);
-  const int k = 2 * (threadIdx.x & 31);
-  if (k < p.m) c[k * B + b] = make_double2(beta0 * fma(f.x, y0.x, -f.y * y0.y), beta0 * fma(f.x, y0.y, f.y * y0.x));
-  if (k + 1 < p.m)
-    c[(k + 1) * B + b] = make_double2(beta0 * fma(f.x, y1.x, -f.y * y1.y), beta0 * fma(f.x, y1.y, f.y * y1.x));
-}
-
-// Convergence check of column b (one warp): the estimate at s_target; if it passes, the column
-// accepts s_target and its coefficients go to c; else, in the basis' last check, the largest
-// step that passes (0 in earlier checks, where only the whole step counts).  The last block to
-// finish takes the minimum over the columns.
+// Convergence check of column b = blockIdx.x (see check_core).  The last block to finish takes the
+// minimum over the columns.
 __device__ void check_column(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
                              const double* __restrict__ beta0, double zr, double zi, double s_target, double tol, int last,
                              const int* st_apply, int* status, double* sb, double2* c, CheckRec* rec) {
-  extern __shared__ double smd[];
+  extern __shared__ __align__(16) double smd[];
   __shared__ int ticket;
   const int b = blockIdx.x;
-  const double bl = beta[(m - 1) * B + b];
-  const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
-  const double2 w = make_double2(s_target * zr * p.r, s_target * zi * p.r);
-  const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
-  double s;
-  if (aw <= cheb::kMaxW) {
-    double2* ck = reinterpret_cast<double2*>(smd);
-    double* first = smd + 2 * (cheb::kMaxTerms + 1);
-    double* lastv = first + cheb::kMaxTerms + 1;
-    const int K = cheb::terms(aw), K2 = last ? max(K, cheb::terms(2.0 * fabs(w.x))) : K;
-    cheb::coefs(w, K, ck);
-    double2 y0, y1;
-    cheb::sum(p, K, K2, ck, y0, y1, last ? first : nullptr, last ? lastv : nullptr);
-    if (cheb::estimate(p, bl, y0, y1) <= tol) {
-      s = s_target;
-      put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
-    } else {
-      s = last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv) : 0.0;
-      if (threadIdx.x == 0) atomicOr(&status[2], 1);
-    }
-  } else {
-    double *d, *q0, *qm;
-    const bool ok = eig_column<false>(m, B, b, alpha, beta, smd, &d, &q0, &qm);
-    if (!ok && threadIdx.x == 0) atomicOr(status, 2);
-    if (last) s = select_step(m, d, q0, qm, bl, s_target, tol, zr, zi);
-    else s = step_error(m, d, q0, qm, bl, s_target, zr, zi) <= tol ? s_target : 0.0;
-    if (threadIdx.x == 0) atomicOr(&status[2], 1);
-  }
+  bool have;
+  const double s = check_core(m, B, b, alpha, beta, beta0, zr, zi, s_target, tol, last, status, smd, c, &have);
   if (threadIdx.x == 0) {
+    if (!have) atomicOr(&status[2], 1);
     sb[b] = s;
     __threadfence();
     ticket = atomicAdd(&status[3], 1);
@@ -499,6 +426,7 @@ __device__ void check_column(int m, int B, const double* __restrict__ alpha, con
     rec->status = atomicAdd(&status[0], 0);
     rec->apply = *st_apply;
     rec->have_c = atomicAdd(&status[2], 0) == 0;
+    rec->m = m;
     status[2] = status[3] = 0;
   }
 }
@@ -511,14 +439,12 @@ __global__ void __launch_bounds__(32) k_krylov_check(int m, int B, const double*
   check_column(m, B, alpha, beta, beta0, zr, zi, s_target, tol, last, st_apply, status, sb, c, rec);
 }
 
-inline size_t check_smem(int m) {
-  return std::max(sizeof(double) * 4 * size_t(m), (cheb::kMaxTerms + 1) * (sizeof(double2) + 2 * sizeof(double)));
-}
+inline size_t check_smem() { return kCheckDoubles * sizeof(double); }
 
 // c[k*B + b] = beta0_b (e^{s z T_b} e_1)_k, one warp per column.
 __device__ void coef_column(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
                             const double* __restrict__ beta0, double zr, double zi, double s, int* status, double2* c) {
-  extern __shared__ double smd[];
+  extern __shared__ __align__(16) double smd[];
   const int b = blockIdx.x;
   const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
   const double2 w = make_double2(s * zr * p.r, s * zi * p.r);
@@ -564,7 +490,7 @@ inline size_t coef_smem(int m) {
 // theta, Q of the eigendecomposition and c = beta0 Q e^{z theta} Q^T e_1 (syk_tridiag_expm)
 __global__ void k_tridiag_eig(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
                               double* __restrict__ theta, double* __restrict__ Qout, int* status) {
-  extern __shared__ double smd[];
+  extern __shared__ __align__(16) double smd[];
   const int b = blockIdx.x, lane = threadIdx.x;
   double *d, *q0, *qm;
   if (!eig_column<true>(m, B, b, alpha, beta, smd, &d, &q0, &qm) && lane == 0) atomicOr(status, 2);
@@ -1040,6 +966,22 @@ std::vector<int> segment_ends(int m, const CheckPlan& pl) {
   return e;
 }
 
+int check_status(const CheckRec& rec) {
+  if (rec.status & 1) {
+    set_error("expmv: non-finite Lanczos scalar");
+    return SYK_ENUMERIC;
+  }
+  if (rec.status & 2) {
+    set_error("expmv: tridiagonal eigensolver did not converge");
+    return SYK_ENUMERIC;
+  }
+  if (rec.apply & 4) {
+    set_error("apply_H: a bounded wait for a staged tile gave up");
+    return SYK_ETIMEOUT;
+  }
+  return SYK_OK;
+}
+
 // outs[k] = e^{fr[k] z H} psi for 0 < fr[0] < ... < fr[nf-1]: the step to fr[nf-1] is split
 // into Krylov bases as the error estimate allows, and each output is combined from the basis
 // whose step covers its fraction.  Restarts pass through outs[nf-1], written last.
@@ -1061,6 +1003,7 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
   CheckRec* rec = static_cast<CheckRec*>(ws.host_stage ? ws.host_stage : pinned_scratch(64));
   SYK_CUDA_CHECK(cudaMemsetAsync(ws.status, 0, sizeof(int) * 4, st));
   double s_rem = fr[nf - 1], s_done = 0.0;
+  bool small = small_basis_applies(P, ws);
   int steps = 0, next = 0;
   const void* cur = psi;
   while (s_rem > 0.0) {
@@ -1069,20 +1012,35 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
       set_error("expmv: more than 100000 Krylov steps");
       return SYK_ENUMERIC;
     }
+    int m_eff = m;
+    const std::vector<int>& ends = steps == 1 ? ends_first : ends_restart;
+    if (small) {  // the whole basis in one launch, up to the check that accepts it
+      const int src = launch_small_basis(P, dtype, ws, orth, two_pass, bt, cur, z, s_rem, tol, ends, st);
+      if (src < 0) return src;
+      if (src > 0) {  // its tables are not there and must not be built now
+        small = false;
+        --steps;
+        continue;
+      }
+      SYK_CUDA_CHECK(cudaMemcpyAsync(rec, ws.rec, sizeof(CheckRec), cudaMemcpyDeviceToHost, st));
+      SYK_CUDA_CHECK(cudaStreamSynchronize(st));
+      m_eff = rec->m;
+      count_applies(B * m_eff);
+      for (int k = 0; k < m_eff; ++k) count_matvec(kMvRows);
+      SYK_TRY(check_status(*rec));
+    } else {
     // v_0 = cur / ||cur||
     Ops<R>::dots(ws, 1, cur, 0, cur, st);
     reduce_parts(ws, 1, ws.h1, st);
     k_norm_init<<<(int(B) + 127) / 128, 128, 0, st>>>(int(B), ws.h1, ws.beta0, ws.inv, ws.sc, ws.status);
     count_launch();
     Ops<R>::scale(ws, cur, ws.vec(0), ws.inv, st);
-    int m_eff = m;
     // Lanczos iterations j in [j0, j1) between two convergence checks
     auto segment = [&](int j0, int j1, cudaStream_t st) -> int {
       // classical Gram-Schmidt against the whole basis; a second pass for FP64 vectors
       for (int j = j0; j < j1; ++j) SYK_TRY(lanczos_step<R>(P, dtype, ws, j, orth, two_pass, bt, st));
       return SYK_OK;
     };
-    const std::vector<int>& ends = steps == 1 ? ends_first : ends_restart;
     int j0 = 0;
     for (size_t si = 0; si < ends.size() && j0 < m; ++si) {
       const int j1 = ends[si];
@@ -1091,31 +1049,21 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
       const bool last = (j1 == m);
       {
         const int mm = j1;
-        k_krylov_check<<<int(B), 32, check_smem(mm), st>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, s_rem, tol,
+        k_krylov_check<<<int(B), 32, check_smem(), st>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, s_rem, tol,
                                                            last ? 1 : 0, P.status, ws.status, ws.sb, ws.c,
                                                            (CheckRec*)ws.rec);
         count_launch();
         SYK_CUDA_CHECK(cudaMemcpyAsync(rec, ws.rec, sizeof(CheckRec), cudaMemcpyDeviceToHost, st));
         SYK_CUDA_CHECK(cudaStreamSynchronize(st));
         prof_collect();
-        if (rec->status & 1) {
-          set_error("expmv: non-finite Lanczos scalar");
-          return SYK_ENUMERIC;
-        }
-        if (rec->status & 2) {
-          set_error("expmv: tridiagonal eigensolver did not converge");
-          return SYK_ENUMERIC;
-        }
-        if (rec->apply & 4) {
-          set_error("apply_H: a bounded wait for a staged tile gave up");
-          return SYK_ETIMEOUT;
-        }
+        SYK_TRY(check_status(*rec));
         if (last || rec->sacc >= s_rem) {
           m_eff = mm;
           break;
         }
       }
       j0 = j1;
+    }
     }
     double s_acc = std::min(rec->sacc, s_rem);
     if (!(s_acc > 1e-13 * s_rem) && !(s_acc >= s_rem)) {
@@ -1335,7 +1283,7 @@ int build_dev_graph(const ApplyParams& P, int dtype, KrylovWS& ws, int orth, boo
     capture_counts_end(&l0, &a0, kinds);
     capture_counts_begin();  // keep counting captured launches away from the global counters
     const int mm = j1;
-    k_krylov_check_dev<<<int(B), 32, check_smem(mm), cs>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, ws.job, ws.ctl,
+    k_krylov_check_dev<<<int(B), 32, check_smem(), cs>>>(mm, int(B), ws.alpha, ws.beta, ws.beta0, ws.job, ws.ctl,
                                                            j1 == m ? 1 : 0, P.status, ws.status, ws.sb, ws.c,
                                                            (CheckRec*)ws.rec);
     const bool has_next = k < ifs.n;
@@ -1462,6 +1410,8 @@ int expmv_chain(const ApplyParams& P_in, int dtype, std::complex<double> z, cons
     return SYK_EINVAL;
   }
   const ApplyParams P = ws.with_split(P_in);
+  // a small sector's basis is one launch already
+  if (small_basis_applies(P, ws)) return expmv_impl(P_in, dtype, z, in, out, B, tol, ws, st, nullptr);
   const int orth = lanczos_orth(dtype);
   const CheckPlan plan = check_plan(P, dtype, ws.D, B, ws.m, z, tol);
   const DevKey key{ws.V, P.m4_tab, P.sector, dtype, B, P.D, ws.m, orth, plan.first, plan.every, graph_epoch()};

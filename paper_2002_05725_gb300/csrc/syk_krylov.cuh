@@ -102,6 +102,13 @@ int expmv_points(const ApplyParams& P, int dtype, std::complex<double> z, const 
 int dot_columns(const void* x, const void* y, int64_t D, int64_t B, int dtype, KrylovWS& ws,
                 double2* res, cudaStream_t st);
 
+// One Krylov basis of a small sector as one launch (syk_small.cu): whether the workspace's shape is
+// one, and the launch, which leaves its result in ws.rec; 1 if its tables are not built and must not
+// be (no_alloc).
+bool small_basis_applies(const ApplyParams& P, const KrylovWS& ws);
+int launch_small_basis(const ApplyParams& P, int dtype, KrylovWS& ws, int orth, bool two_pass, double bt, const void* cur,
+                       std::complex<double> z, double s_rem, double tol, const std::vector<int>& ends, cudaStream_t st);
+
 // Host helpers: pinned staging buffer for small device->host reads.
 void* pinned_scratch(size_t bytes);
 

@@ -296,6 +296,9 @@ extern "C" void syk_free_terms(syk_terms* t) {
       for (void* p : cp)
         if (p) cudaFree(p);
     }
+    void* sp[] = {t->small_dev.coef[0], t->small_dev.coef[1], t->small_dev.flips};
+    for (void* p : sp)
+      if (p) cudaFree(p);
     for (auto& kv : t->block_dev) {
       if (kv.second.chunks) cudaFree(kv.second.chunks);
       if (kv.second.blob) cudaFree(kv.second.blob);
@@ -921,6 +924,56 @@ int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, b
     it = t->block_dev.emplace(key, L).first;
   }
   *out = &it->second;
+  return SYK_OK;
+}
+
+int small_tables(const syk_terms* t, bool may_alloc, const SmallTables** out) {
+  if (may_alloc) SYK_TRY(ensure_device_tables(t));
+  std::lock_guard<std::mutex> lock(t->mtx);
+  SmallTables& S = t->small_dev;
+  if (!S.flips) {
+    if (!may_alloc) return 1;  // not built yet
+    const int n = t->n;
+    const size_t D = size_t(t->D), M = size_t(t->n4) + t->n2 + 1;
+    std::vector<uint32_t> flips(1, 0u);
+    std::vector<std::complex<double>> c[2];
+    for (int sector = 0; sector < 2; ++sector) {
+      c[sector].resize(M * D);
+      for (size_t x = 0; x < D; ++x) {
+        const uint32_t xf = uint32_t(x) | (uint32_t((__builtin_popcount(uint32_t(x)) + sector) & 1) << (n - 1));
+        size_t m = 0;
+        double d = 0.0;
+        for (int a = 0; a < n; ++a)
+          for (int b = a + 1; b < n; ++b)
+            d += ((xf >> a) ^ (xf >> b)) & 1 ? -t->wdiag[size_t(a) * n + b] : t->wdiag[size_t(a) * n + b];
+        c[sector][m++ * D + x] = d;
+        for (int k = 0; k < t->n2; ++k) {
+          const uint32_t* r = &t->m2_rec[4 * size_t(k)];
+          const uint32_t u = ((xf >> (r[2] & 0xff)) & 1) | (((xf >> ((r[2] >> 8) & 0xff)) & 1) << 1);
+          std::complex<double> s = 0.0;
+          for (int q = 0; q < n; ++q) {
+            const double* w = &t->m2_tab[((size_t(k) * n + q) * 4 + u) * 2];
+            s += (xf >> q) & 1 ? -std::complex<double>(w[0], w[1]) : std::complex<double>(w[0], w[1]);
+          }
+          c[sector][m++ * D + x] = __builtin_popcount(r[1] & xf) & 1 ? -s : s;
+        }
+        for (int k = 0; k < t->n4; ++k) {
+          const uint32_t* r = &t->m4_rec[4 * size_t(k)];
+          uint32_t u = (__builtin_popcount(r[1] & xf) & 1) << 4;
+          for (int q = 0; q < 4; ++q) u |= (xf >> ((r[2] >> (8 * q)) & 0xff)) & (1u << q);
+          const double* v = &t->m4_tab[(size_t(k) * 32 + u) * 2];
+          c[sector][m++ * D + x] = std::complex<double>(v[0], v[1]);
+        }
+      }
+    }
+    for (int k = 0; k < t->n2; ++k) flips.push_back(t->m2_rec[4 * size_t(k)]);
+    for (int k = 0; k < t->n4; ++k) flips.push_back(t->m4_rec[4 * size_t(k)]);
+    for (int s = 0; s < 2; ++s)
+      if (!S.coef[s]) SYK_TRY(upload(&S.coef[s], c[s].data(), c[s].size() * 16));
+    S.masks = int(M);
+    SYK_TRY(upload(&S.flips, flips.data(), flips.size() * 4));
+  }
+  *out = &S;
   return SYK_OK;
 }
 

@@ -238,23 +238,23 @@ int launch_epilogue(const ApplyParams& p, void* y, int64_t batch, cudaStream_t s
   return SYK_OK;
 }
 
-// complex64 on the row-block kernel: the tuned shape (variant 4 or 5), or its launch rule where nothing
+// The row-block kernel (complex64; complex128 takes the split copy): the tuned shape (variant 4 or 5), or its launch rule where nothing
 // is tuned; returns 1 if it does not apply.
-int try_block(const ApplyParams& p, const void* psi, void* y, int64_t batch, cudaStream_t st) {
+bool block_choice(const ApplyParams& p, int dtype, int64_t batch, BlockShape* sh) {
   TileChoice tc;
+  if (tile_choice_lookup(p.n * 2, dtype, batch, &tc))
+    return tc.var >= kBlockVariant && block_shape(p.n, batch, dtype, block_rows(tc.var), tc.ntb - 4, tc.cs, sh);
+  return block_default(p.n, batch, dtype, sh);
+}
+int try_block(const ApplyParams& p, int dtype, const void* psi, void* y, int64_t batch, cudaStream_t st) {
   BlockShape sh;
-  if (tile_choice_lookup(p.n * 2, SYK_C64, batch, &tc)) {
-    if (tc.var < kBlockVariant || !block_shape(p.n, batch, block_rows(tc.var), tc.ntb - 4, tc.cs, &sh)) return 1;
-  } else if (!block_default(p.n, batch, &sh)) {
-    return 1;
-  }
-  return launch_apply_block(p, batch, psi, y, st, sh);
+  return block_choice(p, dtype, batch, &sh) ? launch_apply_block(p, batch, psi, y, st, sh) : 1;
 }
 
 template <typename R>
 int launch_apply_T(const ApplyParams& p, const void* psi, void* y, int64_t batch, cudaStream_t st) {
   if constexpr (std::is_same<R, float>::value) {
-    const int rb = try_block(p, psi, y, batch, st);
+    const int rb = try_block(p, SYK_C64, psi, y, batch, st);
     if (rb <= 0) return rb;
   }
   const int rc = try_tiled<R>(p, psi, y, batch, st);
@@ -662,8 +662,9 @@ int launch_apply_df(const ApplyParams& p, const void* psi, void* y, int64_t batc
   const int64_t blocks = std::min<int64_t>((n + threads - 1) / threads, (int64_t)sm_count() * 16);
   k_split_df<<<(unsigned)blocks, threads, 0, st>>>(static_cast<const double2*>(psi), static_cast<float4*>(split), n);
   count_launch();
-  int rc;
-  switch (batch) {
+  // (sectors smaller than the tiled kernel's tiles stay with the FP64 row kernel)
+  int rc = p.D >= (batch == 1 ? 256 : 128) ? try_block(p, SYK_C128, split, y, batch, st) : 1;
+  if (rc > 0) switch (batch) {
     case 1: rc = launch_tiled<DF, 1>(p, split, y, st); break;
     case 2: rc = launch_tiled<DF, 2>(p, split, y, st); break;
     case 4: rc = launch_tiled<DF, 4>(p, split, y, st); break;
@@ -822,7 +823,9 @@ extern "C" int syk_autotune_apply(const syk_terms* terms, int parity, int dtype,
     for (int cs = 1; cs <= 8 && rc == SYK_OK; cs *= 2) {
       if (var >= kBlockVariant) {
         BlockShape sh;
-        if (dtype != SYK_C64 || !block_shape(P.n, batch, block_rows(var), ntb - 4, cs, &sh)) continue;
+        if (!block_shape(P.n, batch, dtype, block_rows(var), ntb - 4, cs, &sh) ||
+            (dtype == SYK_C128 && (c128_arith() != kC128DoubleFloat || P.D < 256)))
+          continue;
       } else {
         if (!coset_var_ok(dtype, batch, var) || (var && !coset_fits(batch, var, ntb))) continue;
         const int rpt = var ? 1 << var : rows_per_thread;
@@ -922,7 +925,9 @@ extern "C" int syk_autotune_import(const char* json) {
     if (num("N", &N) && num("dtype", &dt) && num("batch", &b) && num("ntb", &ntb) && num("cluster", &cs)) {
       num("ms", &ms);
       num("variant", &var);
-      const bool block = (var == kBlockVariant || var == kLastVariant) && dt == SYK_C64 && (b == 1 || b == 2 || b == 4 || b == 8 || b == 16);
+      const bool block = dt == SYK_C64 ? (var == kBlockVariant || var == kLastVariant) &&
+                                             (b == 1 || b == 2 || b == 4 || b == 8 || b == 16)
+                                       : dt == SYK_C128 && var == kLastVariant && (b == 1 || b == 2 || b == 4);
       if (ntb < 6 || ntb > 8 || (cs != 1 && cs != 2 && cs != 4 && cs != 8) ||
           !(block || coset_var_ok(int(dt), int64_t(b), int(var)))) {
         set_error("syk_autotune_import: invalid entry (ntb=%g cluster=%g variant=%g)", ntb, cs, var);

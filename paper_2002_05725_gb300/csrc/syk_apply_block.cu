@@ -17,27 +17,44 @@ int low_bits(int64_t B) {
 
 }  // namespace
 
-int block_aux(int n, int rb) {
+int block_aux(int n, int rb, bool df) {
   const int ng = (n - 1 - rb + 3) / 4;
-  return rb == 5 ? blk::coset_most(5, ng) : blk::coset_most(3, ng);
+  return df ? blk::df_coset_most(3, ng) : rb == 5 ? blk::coset_most(5, ng) : blk::coset_most(3, ng);
 }
 
-size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb) {
+size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb, int elem) {
   const size_t warps = ((size_t(B) << (lb + mb)) + 31) / 32;
-  const size_t share = B == 8 || B == 16 ? warps * (rb == 5 ? blk::share_bytes(5, int(B)) : blk::share_bytes(3, int(B))) : 0;
-  return kStages * ((size_t(B) << (lb + rb + mb)) * 8 + auxb) + 64 + share;
+  const bool df = elem == 16;
+  size_t share = 0;
+  if (B == 8 || B == 16) share = warps * (rb == 5 ? blk::share_bytes(5, int(B)) : blk::share_bytes(3, int(B)));
+  return (df ? 2 : 3) * ((size_t(B) << (lb + rb + mb)) * elem + auxb) + 64 + share;
 }
 
-bool block_shape(int n, int64_t batch, int rb, int mb, int cs, BlockShape* sh) {
-  if (batch < 1 || batch > 32 || mb < 0 || (rb != 3 && rb != 5)) return false;
-  *sh = {rb, low_bits(batch), mb, cs, block_aux(n, rb)};
+bool block_shape(int n, int64_t batch, int dtype, int rb, int mb, int cs, BlockShape* sh) {
+  const bool df = dtype == SYK_C128;
+  if (batch < 1 || batch > 32 || mb < 0 || (rb != 3 && rb != 5) || (df && (rb != 3 || !pow2(batch) || batch > 16))) return false;
+  *sh = {rb, low_bits(batch), mb, cs, block_aux(n, rb, df), df};
   return sh->lb + rb + mb <= n - 1 && (batch << (sh->lb + mb)) <= 256 &&
-         block_smem(batch, sh->lb, rb, mb, sh->auxb) <= kMaxSmemPerCta;
+         block_smem(batch, sh->lb, rb, mb, sh->auxb, df ? 16 : 8) <= kMaxSmemPerCta;
 }
 
-bool block_default(int n, int64_t batch, BlockShape* sh) {
+bool block_default(int n, int64_t batch, int dtype, BlockShape* sh) {
   if (batch < 1 || batch > 32 || n - 1 > 31) return false;
   const int64_t D = int64_t(1) << (n - 1);
+  if (dtype == SYK_C128) {
+    // 1, 2 and 4 states: there the tiled double-float kernel is bound by latency (N = 28, 1 state: 337
+    // us, 140 here; 4 states 255 and 165); with 8 and 16 it is bound by the FP32 operations that both
+    // do and its smaller code wins (N = 36, 16 states: 13.0 ms, 17.0 here).
+    if (batch != 1 && batch != 2 && batch != 4) return false;
+    const int full = 4;  // 256 threads
+    const int64_t ctas = 2 * int64_t(sm_count()), tiles = (D * batch) >> (4 + 3 + full);
+    int cs = 1, mb = full;
+    while (cs < 8 && tiles * cs * 2 <= ctas) cs *= 2;
+    if (cs == 8) mb = 3;
+    for (; mb >= 0; --mb)
+      if (block_shape(n, batch, dtype, 3, mb, cs, sh)) return true;
+    return false;
+  }
   // State counts that are no power of two: sectors below 2^10 stay with the row kernel, which has
   // no waits (N = 24, 6 states: 496 us there, 21 us here).
   if (!pow2(batch) && D < 1024) return false;
@@ -55,10 +72,10 @@ bool block_default(int n, int64_t batch, BlockShape* sh) {
     const int64_t tiles = D >> std::min(n - 1, lb + 5 + full);
     const int mb = tiles >= 25 ? full : full - 1;
     const int cs = tiles >= 100 ? 1 : tiles >= 50 ? 2 : 4;
-    if (block_shape(n, batch, 5, mb, cs, sh)) return true;
+    if (block_shape(n, batch, dtype, 5, mb, cs, sh)) return true;
   }
   for (int mb = std::min(3, full); mb >= 0; --mb)
-    if (block_shape(n, batch, 3, mb, 8, sh)) return true;
+    if (block_shape(n, batch, dtype, 3, mb, 8, sh)) return true;
   return false;
 }
 
@@ -72,17 +89,18 @@ int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, voi
   a.nt = a.SE << sh.mb;
   a.auxb = sh.auxb;
   const BlockLayout* L = nullptr;
-  const int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, !p.no_alloc, &L);
+  const int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, !p.no_alloc, &L);
   if (lr != SYK_OK) return lr > 0 ? 1 : lr;
   for (int k = 0; k < 9; ++k) a.begin[k] = L->begin[k];
   const int which = a.SE != 16 ? kBlockAny : sh.lb == 0 ? kBlock16 : batch == 8 ? kBlockShare : kBlockPow2;
   const bool share = which == kBlock16 || which == kBlockShare;
+  if (sh.df) return launch_block_df(p, a, sh.cs, L, psi, y, st);
   if (sh.rb == 5)
     return share ? launch_block32_share(p, a, which, sh.cs, L, psi, y, st)
                  : launch_block32_direct(p, a, which, sh.cs, L, psi, y, st);
-  return share                 ? launch_block<3, 16, true, true, 256>(p, a, sh.cs, L, psi, y, st)
-         : which == kBlockPow2 ? launch_block<3, 16, true, false, 256>(p, a, sh.cs, L, psi, y, st)
-                               : launch_block<3, 0, true, false, 256>(p, a, sh.cs, L, psi, y, st);
+  return share                 ? launch_block<BlockF32, 3, 16, true, true, 256, 1>(p, a, sh.cs, L, psi, y, st)
+         : which == kBlockPow2 ? launch_block<BlockF32, 3, 16, true, false, 256, 1>(p, a, sh.cs, L, psi, y, st)
+                               : launch_block<BlockF32, 3, 0, true, false, 256, 1>(p, a, sh.cs, L, psi, y, st);
 }
 
 }  // namespace syk

@@ -6,8 +6,8 @@ namespace syk {
 
 int launch_block32_direct(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                           const void* psi, void* y, cudaStream_t st) {
-  return which == kBlockPow2 ? launch_block<5, 16, true, false, 256>(p, a, cs, L, psi, y, st)
-                             : launch_block<5, 0, true, false, 256>(p, a, cs, L, psi, y, st);
+  return which == kBlockPow2 ? launch_block<BlockF32, 5, 16, true, false, 256, 1>(p, a, cs, L, psi, y, st)
+                             : launch_block<BlockF32, 5, 0, true, false, 256, 1>(p, a, cs, L, psi, y, st);
 }
 
 }  // namespace syk

@@ -5,8 +5,8 @@ namespace syk {
 
 int launch_block32_share(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                          const void* psi, void* y, cudaStream_t st) {
-  return which == kBlock16 ? launch_block<5, 16, false, true, 256>(p, a, cs, L, psi, y, st)
-                           : launch_block<5, 16, true, true, 256>(p, a, cs, L, psi, y, st);
+  return which == kBlock16 ? launch_block<BlockF32, 5, 16, false, true, 256, 1>(p, a, cs, L, psi, y, st)
+                           : launch_block<BlockF32, 5, 16, true, true, 256, 1>(p, a, cs, L, psi, y, st);
 }
 
 }  // namespace syk

@@ -35,11 +35,10 @@
 #include <cstdint>
 
 #include "syk_block.cuh"
+#include "syk_block_df.cuh"
 #include "syk_tile.cuh"
 
 namespace syk {
-
-constexpr int kStages = 3;
 
 struct BlockArgs {
   int B, LB, MB;
@@ -49,16 +48,91 @@ struct BlockArgs {
   int begin[9];  // chunk range of each CTA of a tile
 };
 
+// What the kernel does per arithmetic: complex64 with packed FP32 sums, complex128 in double-float.
+template <int RB, bool SHARE>
+struct BlockF32 {
+  using Out = float2;
+  using Sum = float2;
+  using Acc = blk::Acc<RB>;
+  static constexpr int kElem = 8, kRing = 3;
+  static __device__ __forceinline__ void zero(Acc& a) {
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) a.re[r] = a.im[r] = 0ull;
+  }
+  template <int W, bool LOWS>
+  static __device__ __forceinline__ void coset(Acc& a, const blk::CosetAt& at, int stride, const blk::RowCtx& t,
+                                               const ApplyParams&) {
+    blk::coset<RB, W, LOWS, SHARE>(a, at, stride, t);
+  }
+  static __device__ __forceinline__ void record(Acc& a, const unsigned char* prow, int stride, const uint4 rec,
+                                                const unsigned char* tabs, const blk::RowCtx& t) {
+    blk::m2_record<RB, SHARE>(a, prow, stride, rec, tabs, t);
+  }
+  static __device__ __forceinline__ void renorm(Acc&) {}
+  static __device__ __forceinline__ Sum get(const Acc& a, int r) {
+    const float2 x = blk::unpack2(a.re[r]), y = blk::unpack2(a.im[r]);
+    return make_float2(x.x - y.y, x.y + y.x);
+  }
+  static __device__ __forceinline__ void add(Sum& a, const Sum b) {
+    a.x += b.x;
+    a.y += b.y;
+  }
+  static constexpr int share(int B) { return blk::share_bytes(RB, B); }
+};
+template <int RB, bool SHARE>
+struct BlockDf {
+  using Out = double2;
+  using Sum = double2;
+  using Acc = blk::AccDf<RB>;
+  static constexpr int kElem = 16, kRing = 2;
+  static __device__ __forceinline__ void zero(Acc& a) {
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) a.v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  template <int W, bool LOWS>
+  static __device__ __forceinline__ void coset(Acc& a, const blk::CosetAt& at, int stride, const blk::RowCtx& t,
+                                               const ApplyParams& p) {
+    blk::coset_df<RB, W, LOWS>(a, at, stride, t, p.wd_df);
+    if (W < 4) blk::renorm(a);
+  }
+  static __device__ __forceinline__ void record(Acc& a, const unsigned char* prow, int stride, const uint4 rec,
+                                                const unsigned char* tabs, const blk::RowCtx& t) {
+    blk::m2_record_df<RB>(a, prow, stride, rec, tabs, t);
+    blk::renorm(a);
+  }
+  static __device__ __forceinline__ void renorm(Acc& a) { blk::renorm(a); }
+  static __device__ __forceinline__ Sum get(const Acc& a, int r) { return df_to_double2(a.v[r]); }
+  static __device__ __forceinline__ void add(Sum& a, const Sum b) {
+    a.x += b.x;
+    a.y += b.y;
+  }
+  static constexpr int share(int) { return 0; }
+};
+// an element of a CTA of the cluster (8-byte words)
+template <typename T>
+__device__ __forceinline__ T ld_cluster_elem(uint32_t a) {
+  T v;
+  unsigned long long* w = reinterpret_cast<unsigned long long*>(&v);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(T) / 8); ++i)
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(w[i]) : "r"(a + 8u * i) : "memory");
+  return v;
+}
+
 // SEC: SE when known at compile time (16), so that row offsets are immediates; 0 otherwise.
-template <int RB, int SEC, bool LOWB, bool SHARE, int MAXT>
-__global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const BlockArgs c, const int4* __restrict__ chunks,
-                                                      const unsigned char* __restrict__ blob,
-                                                      const float2* __restrict__ psi, float2* __restrict__ y) {
+template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+    k_apply_block(ApplyParams p, const BlockArgs c, const int4* __restrict__ chunks, const unsigned char* __restrict__ blob,
+                  const void* __restrict__ psi, typename Arith<RB, SHARE>::Out* __restrict__ y) {
   using namespace blk;
-  constexpr int R = 1 << RB;
+  using A = Arith<RB, SHARE>;
+  using Out = typename A::Out;
+  using Sum = typename A::Sum;
+  using Real = decltype(Out().x);
+  constexpr int R = 1 << RB, kElem = A::kElem, kStages = A::kRing;
   const int SE = SEC ? SEC : c.SE;
   const int B = c.B, LB = c.LB, MB = c.MB;
-  const int tileb = (SE << (RB + MB)) * 8, stageb = tileb + c.auxb;
+  const int tileb = (SE << (RB + MB)) * kElem, stageb = tileb + c.auxb;
   extern __shared__ __align__(128) unsigned char sm[];
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + kStages * stageb);
   int* done = reinterpret_cast<int*>(full + kStages);  // warps that finished the stage's chunk
@@ -82,11 +156,10 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
   ctx.LB = LB;
   ctx.wd = static_cast<const float*>(p.wd);
   ctx.B = (uint32_t)B;
-  ctx.share = reinterpret_cast<float2*>(sm + kStages * stageb + 64 + (SHARE ? (tid >> 5) * share_bytes(RB, B) : 0));
+  ctx.share = reinterpret_cast<float2*>(sm + kStages * stageb + 64 + (SHARE ? (tid >> 5) * A::share(B) : 0));
 
-  Acc<RB> acc;
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc.re[r] = acc.im[r] = 0ull;
+  typename A::Acc acc;
+  A::zero(acc);
 
   if (tid == 0) {
     for (int k = 0; k < kStages; ++k) {
@@ -122,7 +195,7 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
     constexpr bool LOWS = SEC != 16 || LOWB;
     auto partner = [&](const uint4 rc) SYK_INLINE {  // the thread's partner row 0
       const uint32_t lm = LOWS ? (rc.x >> 16) & 0xffu : 0u;
-      return tb + (size_t)((((uint32_t)mid ^ (rc.x & 0xffffu)) << RB) * SE + ((uint32_t)low ^ lm) * B + s) * 8;
+      return tb + (size_t)((((uint32_t)mid ^ (rc.x & 0xffffu)) << RB) * SE + ((uint32_t)low ^ lm) * B + s) * kElem;
     };
     CosetAt next;
     uint4 rc;
@@ -141,8 +214,10 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
       for (uint32_t k = 0; k < count; ++k) {
         const CosetAt at = next;
         prepare();
-        coset<RB, W, LOWS, SHARE>(acc, at, SE * 8, ctx);
+        A::template coset<W, LOWS>(acc, at, SE * kElem, ctx, p);
+        if (W == 4 && (k & 7u) == 7u) A::renorm(acc);
       }
+      if (W == 4) A::renorm(acc);
     };
     prepare();  // (a record past the last one is never used: it reads the tables behind it)
     run(std::integral_constant<int, 4>{}, cn & 0xffu);
@@ -154,7 +229,7 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
     for (uint32_t k = head.y >> 8; k > 0; --k) {
       const uint4 r2 = rc;
       rc = *rec++;
-      m2_record<RB, SHARE>(acc, partner(r2), SE * 8, r2, cb + r2.w, ctx);
+      A::record(acc, partner(r2), SE * kElem, r2, cb + r2.w, ctx);
     }
     // the warp that finishes the chunk last refills its stage
     __syncwarp();
@@ -179,51 +254,43 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
     __syncthreads();
   }
 
-  // outputs: y[row] = re + i im; the CTAs of a cluster add their sums through shared memory
-  auto value = [&](int r) {
-    const float2 a = unpack2(acc.re[r]), b = unpack2(acc.im[r]);
-    return make_float2(a.x - b.y, a.y + b.x);
-  };
-  const float sc = p.ep_part && p.ep_scale ? (float)p.ep_scale[s] : 1.f;
-  const size_t gbase = (size_t)tile * (tileb / 8);
+  // outputs; the CTAs of a cluster add their sums through shared memory
+  const Real sc = p.ep_part && p.ep_scale ? (Real)p.ep_scale[s] : Real(1);
+  const size_t gbase = (size_t)tile * (tileb / kElem);
   double dr = 0.0, di = 0.0;
-  float fr = 0.f, fi = 0.f;
-  const float2* __restrict__ u = static_cast<const float2*>(p.ep_u);
-  auto emit = [&](size_t e, float2 v, int k) {  // element e of the tile; k counts the thread's elements
+  Real fr = 0, fi = 0;  // flushed to FP64 every 16 elements
+  const Out* __restrict__ u = static_cast<const Out*>(p.ep_u);
+  // element e of the tile; k counts the thread's elements
+  auto emit = [&](size_t e, Out v, int k) {
     if (p.ep_part) {
       v.x *= sc;
       v.y *= sc;
-      const float2 w = u[gbase + e];
-      fr = fmaf(w.x, v.x, fmaf(w.y, v.y, fr));
-      fi = fmaf(w.x, v.y, fmaf(-w.y, v.x, fi));
+      const Out w = u[gbase + e];
+      fr = fma(w.x, v.x, fma(w.y, v.y, fr));
+      fi = fma(w.x, v.y, fma(-w.y, v.x, fi));
       if ((k & 15) == 15) {
         dr += fr;
         di += fi;
-        fr = fi = 0.f;
+        fr = fi = 0;
       }
     }
     y[gbase + e] = v;
   };
   if (csize > 1) {
-    float2* st = reinterpret_cast<float2*>(sm);
+    Sum* st = reinterpret_cast<Sum*>(sm);
     if (active) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) st[((mid << RB) + r) * SE + el] = value(r);
+      for (int r = 0; r < R; ++r) st[((mid << RB) + r) * SE + el] = A::get(acc, r);
     }
     tma::cluster_sync();
     // each CTA adds 1/csize of the tile's elements over the cluster, in rank order
-    const int part = (tileb / 8) / (int)csize;
+    const int part = (tileb / kElem) / (int)csize;
     if (active) {
       int k = 0;
       for (int e = (int)crank * part + tid; e < ((int)crank + 1) * part; e += c.nt, ++k) {
-        float2 v = make_float2(0.f, 0.f);
         const uint32_t a = tma::saddr(st + e);
-        for (uint32_t r = 0; r < csize; ++r) {
-          float2 w;
-          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(w.x), "=f"(w.y) : "r"(tma::map_rank(a, r)) : "memory");
-          v.x += w.x;
-          v.y += w.y;
-        }
+        Sum v = ld_cluster_elem<Sum>(tma::map_rank(a, 0));
+        for (uint32_t r = 1; r < csize; ++r) A::add(v, ld_cluster_elem<Sum>(tma::map_rank(a, r)));
         emit((size_t)e, v, k);
       }
     }
@@ -231,7 +298,7 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
   } else {
     if (active) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) emit((size_t)((mid << RB) + r) * SE + el, value(r), r);
+      for (int r = 0; r < R; ++r) emit((size_t)((mid << RB) + r) * SE + el, A::get(acc, r), r);
     }
     __syncthreads();
   }
@@ -257,10 +324,12 @@ __global__ void __launch_bounds__(MAXT) k_apply_block(ApplyParams p, const Block
 enum { kBlock16 = 0, kBlockShare = 1, kBlockPow2 = 2, kBlockAny = 3 };
 int launch_block32_share(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                          const void* psi, void* y, cudaStream_t st);
+int launch_block_df(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLayout* L, const void* psi, void* y,
+                    cudaStream_t st);
 int launch_block32_direct(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                           const void* psi, void* y, cudaStream_t st);
 
-template <int RB, int SEC, bool LOWB, bool SHARE, int MAXT>
+template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB>
 int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLayout* L, const void* psi, void* y,
              cudaStream_t st) {
   const int tb = a.LB + RB + a.MB;
@@ -269,8 +338,9 @@ int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLa
     set_error("apply_H: %lld CTAs exceed the epilogue buffer (%lld)", (long long)(ntiles * cs), (long long)p.ep_cap);
     return SYK_EINVAL;
   }
-  const size_t smem = block_smem(a.B, a.LB, RB, a.MB, a.auxb);
-  const auto kern = k_apply_block<RB, SEC, LOWB, SHARE, MAXT>;
+  using Out = typename Arith<RB, SHARE>::Out;
+  const size_t smem = block_smem(a.B, a.LB, RB, a.MB, a.auxb, Arith<RB, SHARE>::kElem);
+  const auto kern = k_apply_block<Arith, RB, SEC, LOWB, SHARE, MAXT, MINB>;
   SYK_TRY(ensure_smem_limit((const void*)kern, (int)kMaxSmemPerCta));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ntiles * cs), 1, 1);
@@ -285,9 +355,9 @@ int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLa
   cfg.attrs = attr;
   cfg.numAttrs = cs > 1 ? 1 : 0;
   SYK_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, p, a, (const int4*)L->chunks, (const unsigned char*)L->blob,
-                                    static_cast<const float2*>(psi), static_cast<float2*>(y)));
+                                    psi, static_cast<Out*>(y)));
   count_launch();
-  count_matvec(kMvCoset);
+  count_matvec(Arith<RB, SHARE>::kElem == 8 ? kMvCoset : kMvTiled);
   SYK_CUDA_CHECK(cudaGetLastError());
   return SYK_OK;
 }

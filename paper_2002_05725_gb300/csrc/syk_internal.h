@@ -149,30 +149,33 @@ int launch_coset_var(const ApplyParams& p, int64_t batch, const void* psi, void*
 //   chunks[c] = {h, chunk offset / 16, chunk bytes / 16, 0}; CTA k of a tile has chunks
 //   begin[k] .. begin[k + 1] - 1.  A chunk starts with a 16-byte header: the numbers of cosets
 //   of weight 4, 3, 2, 1 (a byte each), then of weight 0 and of two-spin records (a byte each).
+//   df: tables for double-float arithmetic (syk_block_df.cuh).
 struct BlockHost {
   std::vector<int4> chunks;
   std::vector<unsigned char> blob;
   int begin[9] = {};
 };
-int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, BlockHost* out);
+int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, BlockHost* out);
 struct BlockLayout {
   int4* chunks = nullptr;
   unsigned char* blob = nullptr;
   int begin[9] = {};
 };
-int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool may_alloc, const BlockLayout** out);
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc,
+                 const BlockLayout** out);
 
 // Shape of a row-block launch: rows per thread 2^rb, low and middle bits, CTAs per tile, bytes
 // of a chunk's records and tables.  launch_apply_block returns 1 when the shape does not apply.
 struct BlockShape {
   int rb, lb, mb, cs, auxb;
+  bool df;  // complex128 in double-float
 };
-int block_aux(int n, int rb);  // the smallest auxb
-size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb);
+int block_aux(int n, int rb, bool df);  // the smallest auxb
+size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb, int elem);
 // The shape with 2^rb rows per thread (3 or 5), mb middle bits and cs CTAs per tile, if it exists.
-bool block_shape(int n, int64_t batch, int rb, int mb, int cs, BlockShape* sh);
-// The launch rule of the complex64 matvec; false: the sector is too small, or too many states.
-bool block_default(int n, int64_t batch, BlockShape* sh);
+bool block_shape(int n, int64_t batch, int dtype, int rb, int mb, int cs, BlockShape* sh);
+// The launch rule of the matvec (complex128: double-float); false: the sector is too small, or too many states.
+bool block_default(int n, int64_t batch, int dtype, BlockShape* sh);
 int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, void* y, cudaStream_t st, BlockShape sh);
 
 // Small sectors (syk_small.cu): every mask's coefficient c_m(x) for every row of each sector

@@ -35,6 +35,7 @@
 #include <string>
 
 #include "syk_block.cuh"
+#include "syk_block_df.cuh"
 #include "syk_internal.h"
 
 namespace syk {
@@ -682,21 +683,21 @@ int find_mask(const std::vector<uint32_t>& rec, int count, uint32_t mc) {
 
 // Two-spin tables of mask k (see syk_block.cuh).
 template <int RB>
-void block_m2(const syk_terms* t, int lb, int ng, int k, std::vector<unsigned char>* out) {
+void block_m2(const syk_terms* t, int lb, int ng, int k, bool df, std::vector<unsigned char>* out) {
   using namespace blk;
   const int n = t->n, nb = n - 1;
   std::vector<int> outside;  // spins outside the row bits, top spin excluded
   for (int c = 0; c < nb; ++c)
     if (c < lb || c >= lb + RB) outside.push_back(c);
   std::vector<float> v;
-  v.reserve(4 * size_t(m2_values(RB, ng)) * 2);
   auto W = [&](int c, int u) {
     const double* w = &t->m2_tab[((size_t(k) * n + c) * 4 + u) * 2];
     return std::complex<double>(w[0], w[1]);
   };
   auto put = [&](std::complex<double> c) {
-    v.push_back(float(c.real()));
-    v.push_back(float(c.imag()));
+    const float re = float(c.real()), im = float(c.imag());
+    v.insert(v.end(), {re, im});
+    if (df) v.insert(v.end(), {float(c.real() - double(re)), float(c.imag() - double(im))});
   };
   for (int u = 0; u < 4; ++u) {
     for (int g = 0; g < ng; ++g)
@@ -715,20 +716,19 @@ void block_m2(const syk_terms* t, int lb, int ng, int k, std::vector<unsigned ch
     put(W(nb, u));
   }
   const size_t b0 = out->size();
-  out->resize(b0 + m2_bytes(RB, ng), 0);
+  out->resize(b0 + (df ? df_m2_bytes(RB, ng) : m2_bytes(RB, ng)), 0);
   std::memcpy(out->data() + b0, v.data(), v.size() * 4);
 }
 
 // Appends the tables of the coset with flip `key` outside the row bits (see syk_block.cuh).
 template <int RB>
-void block_tables(const syk_terms* t, int lb, int ng, uint32_t key, int W, std::vector<unsigned char>* blob) {
+void block_tables(const syk_terms* t, int lb, int ng, uint32_t key, int W, bool df, std::vector<unsigned char>* blob) {
   using namespace blk;
   const int lam = __builtin_popcount(key & ((1u << lb) - 1u));
   const uint32_t above_u = uint32_t(((1 << W) - 1) & ~((1 << lam) - 1));  // support bits above the row bits
   const int E = coset_entries(RB, W);
   const size_t b0 = blob->size();
-  blob->resize(b0 + (size_t(E) << W) * kEntryBytes);
-  float* tab = reinterpret_cast<float*>(blob->data() + b0);
+  blob->resize(b0 + (size_t(E) << W) * (df ? kDfEntryBytes : kEntryBytes));
   int at = 0;
   for (uint32_t lo = 0; lo < (1u << RB); ++lo) {
     const int kind = mask_kind(W, lo);
@@ -744,19 +744,23 @@ void block_tables(const syk_terms* t, int lb, int ng, uint32_t key, int W, std::
           int sign = (lam & 1) && ((__builtin_popcount(ul) + K) & 1);
           if (tops == 2) sign ^= __builtin_popcount(un & above_u) & 1;
           const double* v = &t->m4_tab[(size_t(m) * 32 + u + (sign ? 16 : 0)) * 2];
-          float* e = tab + (size_t(un) * E + at + ul * tops + tp) * 4;
-          e[0] = float(v[0]);
-          e[1] = float(v[1]);
-          e[2] = -e[0];
-          e[3] = -e[1];
+          unsigned char* to = blob->data() + b0 + (size_t(un) * E + at + ul * tops + tp) * (df ? kDfEntryBytes : kEntryBytes);
+          const int half = df ? 4 : 2;
+          float q[8] = {float(v[0]), float(v[1])};
+          if (df) {
+            q[2] = float(v[0] - double(q[0]));
+            q[3] = float(v[1] - double(q[1]));
+          }
+          for (int i = 0; i < half; ++i) q[half + i] = -q[i];
+          std::memcpy(to, q, 2 * half * sizeof(float));
         }
     at += tops << K;
   }
-  if (W == 2) block_m2<RB>(t, lb, ng, find_mask(t->m2_rec, t->n2, key), blob);
+  if (W == 2 && !df) block_m2<RB>(t, lb, ng, find_mask(t->m2_rec, t->n2, key), df, blob);
 }
 
 template <int RB>
-int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHost* out) {
+int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, bool df, BlockHost* out) {
   using namespace blk;
   const int nb = t->n - 1, tb = lb + RB + mb, ng = (nb - RB + 3) / 4;
   constexpr int kM2Rec = 5;  // items: cosets by weight, and two-spin records
@@ -778,7 +782,14 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
     for (uint32_t lo = 0; lo < (1u << RB); ++lo) masks += mask_kind(type, lo) == kM4 || mask_kind(type, lo) == kM4Top;
     return masks + 1.0;
   };
-  auto bytes_of = [ng](int type) {
+  auto bytes_of = [ng, df](int type) {
+    if (df)
+      return type == 4   ? df_coset_bytes(RB, 4)
+             : type == 3 ? df_coset_bytes(RB, 3)
+             : type == 2 ? df_coset_bytes(RB, 2)
+             : type == 1 ? df_coset_bytes(RB, 1)
+             : type == 0 ? df_coset_bytes(RB, 0)
+                         : df_m2_bytes(RB, ng);
     return type == 4   ? coset_bytes(RB, 4, ng)
            : type == 3 ? coset_bytes(RB, 3, ng)
            : type == 2 ? coset_bytes(RB, 2, ng)
@@ -786,7 +797,7 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
            : type == 0 ? coset_bytes(RB, 0, ng)
                        : m2_bytes(RB, ng);
   };
-  const double fill = 4.0;
+  const double fill = df ? 0.7 : 4.0;
   std::vector<Chunk> all;
   const uint32_t nlow = 1u << lb, nmid = 1u << mb;
   for (uint32_t h = 0; h < (1u << (nb - tb)); ++h) {
@@ -798,7 +809,7 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
         const int W = wh + __builtin_popcount(m) + __builtin_popcount(l);
         const uint32_t key = (h << tb) | (m << (lb + RB)) | l;
         if (W <= 4) items.push_back({W, key});
-        if (W <= 1)
+        if (W <= (df ? 2 : 1))
           for (uint32_t lo = 0; lo < (1u << RB); ++lo)
             if (mask_kind(W, lo) == kM2 || mask_kind(W, lo) == kM2Top) items.push_back({kM2Rec, key | (lo << lb)});
       }
@@ -855,7 +866,7 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
           rec.x |= lo << 24;
           rec.y = t->m2_rec[4 * size_t(m) + 1];
           rec.z = t->m2_rec[4 * size_t(m) + 2];
-          block_m2<RB>(t, lb, ng, m, &out->blob);
+          block_m2<RB>(t, lb, ng, m, df, &out->blob);
         } else {
           const int W = c.items[e].type;
           rec.x |= uint32_t(__builtin_popcount(low) & 1) << 31;
@@ -870,7 +881,7 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
             }
           }
           for (int q = below; q < 4; ++q) rec.z |= 31u << (8 * q);
-          block_tables<RB>(t, lb, ng, key, W, &out->blob);
+          block_tables<RB>(t, lb, ng, key, W, df, &out->blob);
         }
         std::memcpy(out->blob.data() + b0 + 16 + 16 * e, &rec, 16);
       }
@@ -883,18 +894,14 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, BlockHo
 
 }  // namespace
 
-int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, BlockHost* out) {
-  if (rb < 3 || rb > 5 || lb < 0 || lb > 8 || mb < 0 || mb > 15 || cs < 1 || cs > 8 || lb + rb + mb > t->n - 1) {
+int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, BlockHost* out) {
+  if ((rb != 3 && rb != 5) || (df && rb != 3) || lb < 0 || lb > 8 || mb < 0 || mb > 15 || cs < 1 || cs > 8 || lb + rb + mb > t->n - 1) {
     set_error("block_layout: unsupported shape (rb=%d lb=%d mb=%d cs=%d)", rb, lb, mb, cs);
     return SYK_EINVAL;
   }
   *out = BlockHost();
   try {
-    switch (rb) {
-      case 3: return block_layout_T<3>(t, lb, mb, cs, auxb, out);
-      case 4: return block_layout_T<4>(t, lb, mb, cs, auxb, out);
-      default: return block_layout_T<5>(t, lb, mb, cs, auxb, out);
-    }
+    return rb == 3 ? block_layout_T<3>(t, lb, mb, cs, auxb, df, out) : block_layout_T<5>(t, lb, mb, cs, auxb, df, out);
   } catch (const std::bad_alloc&) {
     set_error("block_layout: out of host memory");
     return SYK_ENOMEM;
@@ -904,15 +911,17 @@ int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int au
   }
 }
 
-int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool may_alloc, const BlockLayout** out) {
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc,
+                 const BlockLayout** out) {
   if (may_alloc) SYK_TRY(ensure_device_tables(t));
   std::lock_guard<std::mutex> lock(t->mtx);
-  const uint64_t key = uint64_t(rb) | uint64_t(lb) << 8 | uint64_t(mb) << 16 | uint64_t(cs) << 24 | uint64_t(auxb) << 32;
+  const uint64_t key = uint64_t(rb) | uint64_t(lb) << 8 | uint64_t(mb) << 16 | uint64_t(cs) << 24 |
+                       uint64_t(df ? 1 : 0) << 28 | uint64_t(auxb) << 32;
   auto it = t->block_dev.find(key);
   if (it == t->block_dev.end()) {
     if (!may_alloc) return 1;  // not built yet
     BlockHost H;
-    SYK_TRY(block_layout_host(t, rb, lb, mb, cs, auxb, &H));
+    SYK_TRY(block_layout_host(t, rb, lb, mb, cs, auxb, df, &H));
     BlockLayout L;
     std::memcpy(L.begin, H.begin, sizeof(L.begin));
     SYK_TRY(upload(&L.chunks, H.chunks.data(), H.chunks.size() * sizeof(int4)));

@@ -22,6 +22,7 @@
 
 #include "syk_krylov.cuh"
 #include "syk_tile.cuh"
+#include "syk_check.cuh"
 #include "syk_tridiag.cuh"
 
 namespace syk {
@@ -88,7 +89,7 @@ struct PArgs {
 };
 
 struct PCtl {
-  int item, status, first;
+  int item, status, first, miss;
   double s_acc;
 };
 
@@ -386,7 +387,9 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
   const int D = it.D, m = a.m, tid = threadIdx.x;
   const double tol = a.tol;
   const size_t fstride = (size_t)m * m + 4 * (size_t)m + 2;  // doubles per column: Q, d, e, fg, rot
-  const bool fused = a.L.ncol >= B;
+  // terms of the check's expansion that fit a column's share of region A (which holds at least 4m
+  // doubles a column)
+  const int cap = min(cheb::kMaxTerms, (a.L.rec - a.L.A) / (B * 32) - 1);
   if (zr == 0.0 && zi == 0.0) {
     if (out != in) cta_copy<B>(in, out, D);
     return;
@@ -520,47 +523,23 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
         }
         __syncthreads();
       }
-      // convergence check on T of dimension j1: warp b checks column b.  Fused (every column's
-      // eigenvector matrix fits region A at once): the check runs the full eigendecomposition,
-      // and the accepted basis takes its coefficients from it (on GB300 the FP64-bound
-      // rows-only and full eigensolves cost about the same); otherwise rows 0 and j1-1 only.
+      // convergence check on T of dimension j1: warp b checks column b (check_core), with an equal
+      // share of region A for the terms of its expansion; a column that accepts what remains leaves
+      // its combination coefficients in cc
       {
         const long long t0 = clk();
         const int wp = tid >> 5, lane = tid & 31;
+        if (tid == 0) S.ctl->miss = 0;
+        __syncthreads();
         if (wp < B) {
-          const int b = wp;
-          double *d, *e, *q0, *qm;
-          bool ok = true;
-          if (fused) {
-            double* Qm = reinterpret_cast<double*>(S.A) + (size_t)b * fstride;
-            d = Qm + (size_t)m * m;
-            e = d + m;
-            for (int k = lane; k < j1; k += 32) {
-              d[k] = S.alpha[k * B + b];
-              e[k] = k + 1 < j1 ? S.beta[k * B + b] : 0.0;
-            }
-            __syncwarp();
-            ok = tridiag_eig_warp(j1, d, e, Qm, e + 3 * m);
-            q0 = Qm;
-            qm = Qm + (size_t)(j1 - 1) * j1;
-          } else {
-            d = reinterpret_cast<double*>(S.A) + (size_t)b * 4 * m;
-            e = d + m;
-            q0 = e + m;
-            qm = q0 + m;
-            for (int k = lane; k < j1; k += 32) {
-              d[k] = S.alpha[k * B + b];
-              e[k] = k + 1 < j1 ? S.beta[k * B + b] : 0.0;
-            }
-            __syncwarp();
-            if (lane == 0) ok = tridiag_eig_rows(j1, d, e, q0, qm);
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            __syncwarp();
+          bool have;
+          const double s = check_core(j1, B, wp, S.alpha, S.beta, S.beta0, zr, zi, s_rem, tol, j1 == m, &S.ctl->status,
+                                      reinterpret_cast<double*>(S.A) + (size_t)wp * 4 * (cap + 1), S.cc, &have, cap,
+                                      1.0 / (1 << kBisect));
+          if (lane == 0) {
+            S.sb[wp] = s;
+            if (!have) S.ctl->miss = 1;
           }
-          if (!ok && lane == 0) atomicOr(&S.ctl->status, 2);
-          const double bl = S.beta[(j1 - 1) * B + b];
-          const double s = select_step(j1, d, q0, qm, bl, s_rem, tol, zr, zi, kBisect);
-          if (lane == 0) S.sb[b] = s;
         }
         __syncthreads();
         if (tid == 0) {
@@ -588,13 +567,19 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
       return;
     }
     const bool final_basis = s_acc >= s_rem || s_done + s_acc * (1.0 + 1e-13) >= 1.0;
-    // full eigendecomposition of the accepted basis (unless the last check made it) and the
-    // combination coefficients
-    //   cc[k][b] = beta0_b sum_l Q_b[k][l] e^{s_acc z theta_l} Q_b[0][l]   (as k_tridiag_coef)
-    {
+    // the combination coefficients cc[k][b] = beta0_b (e^{s_acc z T_b} e_1)_k, unless the check left
+    // them: by the expansion, or (more terms than region A holds) the full eigendecomposition
+    if (s_acc < s_rem || S.ctl->miss) {
       const long long t0 = clk();
       const int wp = tid >> 5, lane = tid & 31;
-      for (int r0 = 0; r0 < B; r0 += a.L.ncol) {
+      __syncthreads();
+      if (tid == 0) S.ctl->miss = 0;
+      __syncthreads();
+      if (wp < B && !coefs_core(m_eff, B, wp, S.alpha, S.beta, S.beta0, zr, zi, s_acc,
+                                reinterpret_cast<double*>(S.A) + (size_t)wp * 4 * (cap + 1), S.cc, cap) && lane == 0)
+        S.ctl->miss = 1;
+      __syncthreads();
+      for (int r0 = S.ctl->miss ? 0 : B; r0 < B; r0 += a.L.ncol) {
         const int b = r0 + wp;
         if (wp < a.L.ncol && b < B) {
           double* Qm = reinterpret_cast<double*>(S.A) + (size_t)wp * fstride;
@@ -602,15 +587,13 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
           double* e = d + m;
           double* fg = e + m;     // 2 m doubles
           double* rot = fg + 2 * m;
-          if (!fused) {
-            for (int k = lane; k < m_eff; k += 32) {
-              d[k] = S.alpha[k * B + b];
-              e[k] = k + 1 < m_eff ? S.beta[k * B + b] : 0.0;
-            }
-            __syncwarp();
-            const bool ok = tridiag_eig_warp(m_eff, d, e, Qm, rot);
-            if (!ok && lane == 0) atomicOr(&S.ctl->status, 2);
+          for (int k = lane; k < m_eff; k += 32) {
+            d[k] = S.alpha[k * B + b];
+            e[k] = k + 1 < m_eff ? S.beta[k * B + b] : 0.0;
           }
+          __syncwarp();
+          const bool ok = tridiag_eig_warp(m_eff, d, e, Qm, rot);
+          if (!ok && lane == 0) atomicOr(&S.ctl->status, 2);
           for (int l = lane; l < m_eff; l += 32) {
             const double2 f = cexp_scaled(s_acc, zr, zi, d[l]);
             const double g = Qm[l];  // row 0
@@ -632,7 +615,7 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
         __syncthreads();
       }
       pc.cy[2] += clk() - t0;
-      if (!fused) ++pc.neig;
+      ++pc.neig;
     }
     if (S.ctl->status & 3) return;
     for (int e = tid; e < m_eff * B; e += kPNT) {
@@ -929,13 +912,14 @@ int otoc_batch_persistent(const syk_otoc_item* items, const std::vector<int>& id
     p.D = (int)T->D;
     p.n4 = T->n4;
     p.n2 = T->n2;
-    // Check plan from the measured costs in this kernel: a convergence check (FP64 eigensolves
-    // of Bs columns sharing the SM's FP64 pipe) ~0.6 + 0.05 Bs ms; a matvec ~(0.10 + 0.035 Bs)
-    // ns per row x mask pair.  The later checks come every ~sqrt(16 ratio) vectors (the
-    // expected overshoot of a few vectors against the checks saved), the first at 3/4 of the
-    // predicted dimension when checks are cheap, 7/8 or all of it when they are not.
+    // Check plan from the measured costs in this kernel: a convergence check (Bs columns sharing
+    // the SM's FP64 pipe) 0.085 ms at 8 columns (227e6 cycles in 1385 checks; the eigensolves it
+    // replaces: 1.0 ms), ~0.04 + 0.006 Bs; a matvec
+    // ~(0.10 + 0.035 Bs) ns per row x mask pair.  The later checks come every ~sqrt(16 ratio)
+    // vectors (the expected overshoot of a few vectors against the checks saved), the first at 3/4
+    // of the predicted dimension when checks are cheap, 7/8 or all of it when they are not.
     const double mv_ms = double(T->D) * double(T->n4 + T->n2 + 1) * (0.10 + 0.035 * double(Bs)) * 1e-6;
-    const double ratio = (0.6 + 0.05 * double(Bs)) / std::max(mv_ms, 1e-6);
+    const double ratio = (0.04 + 0.006 * double(Bs)) / std::max(mv_ms, 1e-6);
     p.every = std::max(2, std::min(8, (int)std::lround(std::sqrt(16.0 * ratio))));
     p.first8 = ratio < 1.0 ? 6 : ratio < 4.0 ? 7 : 8;
   }

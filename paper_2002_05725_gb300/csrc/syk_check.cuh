@@ -58,23 +58,25 @@ __device__ inline void put_coefs(const cheb::Proj& p, double s, double zr, doubl
 // Convergence check of column b by one warp: the estimate at s_target; if it passes, the column
 // accepts s_target and its coefficients go to c (*have); else, in the basis' last check, the largest
 // step that passes (0 in earlier checks, where only the whole step counts).  Returns the step; error
-// bits go to status[0].  smd: kCheckDoubles doubles of the warp's own.
+// bits go to status[0].  smd: the warp's own scratch for `cap` terms of the expansion, 4 (cap + 1)
+// doubles (at least 4m); beyond cap the eigendecomposition.  narrow: relative width of the step search.
 constexpr int kCheckDoubles = 4 * (cheb::kMaxTerms + 1);
 static_assert(kCheckDoubles >= 4 * SYK_MAX_KRYLOV, "scratch of the eigendecomposition's rows");
 static __device__ double check_core(int m, int B, int b, const double* alpha, const double* beta, const double* beta0,
                                     double zr, double zi, double s_target, double tol, bool last, int* status,
-                                    double* smd, double2* c, bool* have) {
+                                    double* smd, double2* c, bool* have, int cap = cheb::kMaxTerms,
+                                    double narrow = 3e-8) {
   const int lane = threadIdx.x & 31;
   const double bl = beta[(m - 1) * B + b];
   const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
   const double2 w = make_double2(s_target * zr * p.r, s_target * zi * p.r);
   const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
   *have = false;
-  if (aw <= cheb::kMaxW) {
+  const int K = cheb::terms(aw), K2 = last ? max(K, cheb::terms(2.0 * fabs(w.x))) : K;
+  if (aw <= cheb::kMaxW && K2 <= cap) {
     double2* ck = reinterpret_cast<double2*>(smd);
-    double* first = smd + 2 * (cheb::kMaxTerms + 1);
-    double* lastv = first + cheb::kMaxTerms + 1;
-    const int K = cheb::terms(aw), K2 = last ? max(K, cheb::terms(2.0 * fabs(w.x))) : K;
+    double* first = smd + 2 * (cap + 1);
+    double* lastv = first + cap + 1;
     cheb::coefs(w, K, ck);
     double2 y0, y1;
     cheb::sum(p, K, K2, ck, y0, y1, last ? first : nullptr, last ? lastv : nullptr);
@@ -83,13 +85,30 @@ static __device__ double check_core(int m, int B, int b, const double* alpha, co
       *have = true;
       return s_target;
     }
-    return last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv) : 0.0;
+    return last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv, narrow) : 0.0;
   }
   double *d, *q0, *qm;
   const bool ok = eig_column<false>(m, B, b, alpha, beta, smd, &d, &q0, &qm);
   if (!ok && lane == 0) atomicOr(status, 2);
   if (last) return select_step(m, d, q0, qm, bl, s_target, tol, zr, zi);
   return step_error(m, d, q0, qm, bl, s_target, zr, zi) <= tol ? s_target : 0.0;
+}
+
+// The coefficients of column b at the step s by one warp (put_coefs), false when they need more than
+// `cap` terms; smd: 2 (cap + 1) doubles.
+static __device__ bool coefs_core(int m, int B, int b, const double* alpha, const double* beta, const double* beta0,
+                                  double zr, double zi, double s, double* smd, double2* c, int cap = cheb::kMaxTerms) {
+  const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
+  const double2 w = make_double2(s * zr * p.r, s * zi * p.r);
+  const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
+  const int K = cheb::terms(aw);
+  if (aw > cheb::kMaxW || K > cap) return false;
+  double2* ck = reinterpret_cast<double2*>(smd);
+  cheb::coefs(w, K, ck);
+  double2 y0, y1;
+  cheb::sum(p, K, K, ck, y0, y1, nullptr, nullptr);
+  put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
+  return true;
 }
 
 }  // namespace syk

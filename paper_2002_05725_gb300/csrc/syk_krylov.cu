@@ -446,18 +446,7 @@ __device__ void coef_column(int m, int B, const double* __restrict__ alpha, cons
                             const double* __restrict__ beta0, double zr, double zi, double s, int* status, double2* c) {
   extern __shared__ __align__(16) double smd[];
   const int b = blockIdx.x;
-  const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
-  const double2 w = make_double2(s * zr * p.r, s * zi * p.r);
-  const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
-  if (aw <= cheb::kMaxW) {
-    double2* ck = reinterpret_cast<double2*>(smd);
-    const int K = cheb::terms(aw);
-    cheb::coefs(w, K, ck);
-    double2 y0, y1;
-    cheb::sum(p, K, K, ck, y0, y1, nullptr, nullptr);
-    put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
-    return;
-  }
+  if (coefs_core(m, B, b, alpha, beta, beta0, zr, zi, s, smd, c)) return;
   double *d, *q0, *qm;
   if (!eig_column<true>(m, B, b, alpha, beta, smd, &d, &q0, &qm) && threadIdx.x == 0) atomicOr(status, 2);
   for (int k = threadIdx.x; k < m; k += 32) {

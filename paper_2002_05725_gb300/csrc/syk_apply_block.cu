@@ -42,10 +42,12 @@ bool block_default(int n, int64_t batch, int dtype, BlockShape* sh) {
   if (batch < 1 || batch > 32 || n - 1 > 31) return false;
   const int64_t D = int64_t(1) << (n - 1);
   if (dtype == SYK_C128) {
-    // 1, 2 and 4 states: there the tiled double-float kernel is bound by latency (N = 28, 1 state: 337
-    // us, 140 here; 4 states 255 and 165); with 8 and 16 it is bound by the FP32 operations that both
-    // do and its smaller code wins (N = 36, 16 states: 13.0 ms, 17.0 here).
-    if (batch != 1 && batch != 2 && batch != 4) return false;
+    // One state, and 2 and 4 states of sectors up to 2^15 elements: there the tiled double-float
+    // kernel is bound by latency (N = 28: 1 state 337 us, 140 here, 2 states 298 and 156, 4 states 255
+    // and 163; N = 36, 1 state 1.94 and 1.32 ms; N = 40, 1 state 7.7 and 6.8).  Beyond it is bound by
+    // the FP32 operations that both do and its smaller code wins (N = 36, 2 states 2.28 ms, 2.45 here;
+    // 4 states 3.9 and 4.7, 16 states 13.0 and 17.0).
+    if (batch != 1 && !((batch == 2 || batch == 4) && D * batch <= (int64_t(1) << 15))) return false;
     const int full = 4;  // 256 threads
     const int64_t ctas = 2 * int64_t(sm_count()), tiles = (D * batch) >> (4 + 3 + full);
     int cs = 1, mb = full;

@@ -91,7 +91,14 @@ int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, voi
   a.nt = a.SE << sh.mb;
   a.auxb = sh.auxb;
   const BlockLayout* L = nullptr;
-  const int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, !p.no_alloc, &L);
+  int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, false, &L);
+  if (lr > 0 && !p.no_alloc) {
+    // the first launch of a shape builds its layout, which a stream under capture cannot
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    else if (cap == cudaStreamCaptureStatusNone)
+      lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, true, &L);
+  }
   if (lr != SYK_OK) return lr > 0 ? 1 : lr;
   for (int k = 0; k < 9; ++k) a.begin[k] = L->begin[k];
   const int which = a.SE != 16 ? kBlockAny : sh.lb == 0 ? kBlock16 : batch == 8 ? kBlockShare : kBlockPow2;

@@ -81,3 +81,24 @@ def test_larger_sector_rows_and_epilogue(torch, B):
     a = syk.syk_expmv(terms, 0, z, x, krylov_dim=40, tol=1e-7)[0].cpu().numpy()
     b = syk.syk_expmv(terms, 0, z, to_dev(torch, psi, "c128"), krylov_dim=40, tol=1e-12)[0].cpu().numpy()
     assert rel(a, b) < TOL["c64"]
+
+
+def test_first_launch_under_stream_capture(torch):
+    """A state count whose layout is not built yet, first used under stream capture: the row kernel
+    is recorded instead (building a layout allocates), and the replayed graph is correct."""
+    N = 22
+    syk.syk_autotune_reset()
+    J = inputs.couplings(N, 8)
+    terms = syk.syk_build_terms(N, J)
+    H = hm.H_sector_sparse(N, J, 0)
+    _check(torch, N, 4, H, terms, 0)  # uploads the term set
+    psi = inputs.random_states(N, 5, 9)
+    x = to_dev(torch, psi, "c64")
+    y = torch.zeros_like(x)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        syk.syk_apply_H(terms, 0, x, out=y)
+    g.replay()
+    torch.cuda.synchronize()
+    assert rel(y.cpu().numpy(), H @ psi.T) < TOL["c64"]
+    _check(torch, N, 5, H, terms, 0)

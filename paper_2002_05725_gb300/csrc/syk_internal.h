@@ -157,7 +157,7 @@ struct BlockHost {
 };
 int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, BlockHost* out);
 struct BlockLayout {
-  int4* chunks = nullptr;
+  int4* chunks = nullptr;  // in blob's allocation, behind the tables
   unsigned char* blob = nullptr;
   int begin[9] = {};
 };

@@ -301,7 +301,6 @@ extern "C" void syk_free_terms(syk_terms* t) {
     for (void* p : sp)
       if (p) cudaFree(p);
     for (auto& kv : t->block_dev) {
-      if (kv.second.chunks) cudaFree(kv.second.chunks);
       if (kv.second.blob) cudaFree(kv.second.blob);
     }
     if (prev >= 0) cudaSetDevice(prev);
@@ -689,35 +688,47 @@ void block_m2(const syk_terms* t, int lb, int ng, int k, bool df, std::vector<un
   std::vector<int> outside;  // spins outside the row bits, top spin excluded
   for (int c = 0; c < nb; ++c)
     if (c < lb || c >= lb + RB) outside.push_back(c);
-  std::vector<float> v;
+  const size_t b0 = out->size();
+  out->resize(b0 + (df ? df_m2_bytes(RB, ng) : m2_bytes(RB, ng)), 0);
+  float* v = reinterpret_cast<float*>(out->data() + b0);
   auto W = [&](int c, int u) {
     const double* w = &t->m2_tab[((size_t(k) * n + c) * 4 + u) * 2];
     return std::complex<double>(w[0], w[1]);
   };
   auto put = [&](std::complex<double> c) {
     const float re = float(c.real()), im = float(c.imag());
-    v.insert(v.end(), {re, im});
-    if (df) v.insert(v.end(), {float(c.real() - double(re)), float(c.imag() - double(im))});
-  };
-  for (int u = 0; u < 4; ++u) {
-    for (int g = 0; g < ng; ++g)
-      for (int e = 0; e < 16; ++e) {
-        std::complex<double> s = 0.0;
-        for (int b = 0; b < 4; ++b)
-          if (size_t(4 * g + b) < outside.size()) s += ((e >> b) & 1) ? -W(outside[4 * g + b], u) : W(outside[4 * g + b], u);
-        put(s);
-      }
-    for (int r = 0; r < (1 << RB); ++r) {
-      std::complex<double> s = 0.0;
-      for (int b = 0; b < RB; ++b) s += ((r >> b) & 1) ? -W(lb + b, u) : W(lb + b, u);
-      put(s);
+    *v++ = re;
+    *v++ = im;
+    if (df) {
+      *v++ = float(c.real() - double(re));
+      *v++ = float(c.imag() - double(im));
     }
+  };
+  // sums over the sign patterns of the spins c[0..cnt): s[e] takes c[b] with - where bit b of e is set
+  std::complex<double> s[1 << (RB > 4 ? RB : 4)];
+  auto sums = [&](const int* c, int cnt, int u) {
+    s[0] = 0.0;
+    for (int b = 0; b < cnt; ++b) {
+      const std::complex<double> w = W(c[b], u);
+      for (int e = 0; e < (1 << b); ++e) {
+        s[e | (1 << b)] = s[e] - w;
+        s[e] += w;
+      }
+    }
+  };
+  int rows[RB];
+  for (int b = 0; b < RB; ++b) rows[b] = lb + b;
+  for (int u = 0; u < 4; ++u) {
+    for (int g = 0; g < ng; ++g) {
+      const int cnt = std::min(4, int(outside.size()) - 4 * g);
+      sums(outside.data() + 4 * g, cnt, u);
+      for (int e = 0; e < 16; ++e) put(s[e & ((1 << cnt) - 1)]);
+    }
+    sums(rows, RB, u);
+    for (int r = 0; r < (1 << RB); ++r) put(s[r]);
     for (int b = 0; b < RB; ++b) put(W(lb + b, u));
     put(W(nb, u));
   }
-  const size_t b0 = out->size();
-  out->resize(b0 + (df ? df_m2_bytes(RB, ng) : m2_bytes(RB, ng)), 0);
-  std::memcpy(out->data() + b0, v.data(), v.size() * 4);
 }
 
 // Appends the tables of the coset with flip `key` outside the row bits (see syk_block.cuh).
@@ -736,24 +747,29 @@ void block_tables(const syk_terms* t, int lb, int ng, uint32_t key, int W, bool 
     if (kind != kM4 && kind != kM4Top) continue;
     const int m = find_mask(t->m4_rec, t->n4, mc);
     const int K = __builtin_popcount(lo), tops = kind == kM4Top ? 2 : 1;
-    for (uint32_t un = 0; un < (1u << W); ++un)
-      for (uint32_t ul = 0; ul < (1u << K); ++ul)
-        for (int tp = 0; tp < tops; ++tp) {
-          // support bits in ascending spin order: low bits, row bits, bits above, top spin
-          const uint32_t u = (un & ((1u << lam) - 1u)) | (ul << lam) | ((un >> lam) << (lam + K)) | (uint32_t(tp) << (W + K));
-          int sign = (lam & 1) && ((__builtin_popcount(ul) + K) & 1);
-          if (tops == 2) sign ^= __builtin_popcount(un & above_u) & 1;
-          const double* v = &t->m4_tab[(size_t(m) * 32 + u + (sign ? 16 : 0)) * 2];
-          unsigned char* to = blob->data() + b0 + (size_t(un) * E + at + ul * tops + tp) * (df ? kDfEntryBytes : kEntryBytes);
-          const int half = df ? 4 : 2;
-          float q[8] = {float(v[0]), float(v[1])};
+    const size_t eb = df ? kDfEntryBytes : kEntryBytes;
+    const double* tab = &t->m4_tab[size_t(m) * 64];
+    for (uint32_t un = 0; un < (1u << W); ++un) {
+      // support bits in ascending spin order: low bits, row bits, bits above, top spin
+      const uint32_t u0 = (un & ((1u << lam) - 1u)) | ((un >> lam) << (lam + K));
+      const int flip = tops == 2 ? __builtin_popcount(un & above_u) & 1 : 0;
+      unsigned char* to = blob->data() + b0 + (size_t(un) * E + at) * eb;
+      for (uint32_t ul = 0; ul < (1u << K); ++ul) {
+        const int sign = flip ^ (lam & (__builtin_popcount(ul) + K) & 1);
+        for (int tp = 0; tp < tops; ++tp, to += eb) {
+          const double* v = tab + 2 * size_t((u0 | (ul << lam) | (uint32_t(tp) << (W + K))) + (sign ? 16 : 0));
+          const float re = float(v[0]), im = float(v[1]);
           if (df) {
-            q[2] = float(v[0] - double(q[0]));
-            q[3] = float(v[1] - double(q[1]));
+            const float rl = float(v[0] - double(re)), il = float(v[1] - double(im));
+            const float q[8] = {re, im, rl, il, -re, -im, -rl, -il};
+            std::memcpy(to, q, sizeof(q));
+          } else {
+            const float q[4] = {re, im, -re, -im};
+            std::memcpy(to, q, sizeof(q));
           }
-          for (int i = 0; i < half; ++i) q[half + i] = -q[i];
-          std::memcpy(to, q, 2 * half * sizeof(float));
         }
+      }
+    }
     at += tops << K;
   }
   if (W == 2 && !df) block_m2<RB>(t, lb, ng, find_mask(t->m2_rec, t->n2, key), df, blob);
@@ -770,10 +786,12 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, bool df
   };
   struct Chunk {
     uint32_t h;
-    std::vector<Item> items;  // cosets of weight 4, 3, 2, 1, 0, then two-spin records
+    size_t first = 0;  // its items in the pool: cosets of weight 4, 3, 2, 1, 0, then two-spin records
+    size_t n = 0;
     int count[6] = {};
     double cost = 0.0;
   };
+  std::vector<Item> pool;  // every chunk's items, chunk after chunk
   // arithmetic of an item in units of one mask: its masks, the partner-row loads and, for
   // two-spin masks, their coefficients; a tile's copy takes about as long as 4 masks
   auto cost_of = [](int type) {
@@ -800,37 +818,46 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, bool df
   const double fill = df ? 0.7 : 4.0;
   std::vector<Chunk> all;
   const uint32_t nlow = 1u << lb, nmid = 1u << mb;
+  std::vector<uint32_t> by[5];  // flips of the middle and low bits by their weight
+  for (uint32_t m = 0; m < nmid; ++m)
+    for (uint32_t l = 0; l < nlow; ++l) {
+      const int w = __builtin_popcount(m) + __builtin_popcount(l);
+      if (w <= 4) by[w].push_back((m << (lb + RB)) | l);
+    }
+  const int most2 = df ? 2 : 1;  // two-spin records of their own: cosets up to this weight
+  std::vector<uint32_t> upto[3];
+  for (int w = 0; w <= most2; ++w) {
+    for (int v = 0; v <= w; ++v) upto[w].insert(upto[w].end(), by[v].begin(), by[v].end());
+    std::sort(upto[w].begin(), upto[w].end());
+  }
   for (uint32_t h = 0; h < (1u << (nb - tb)); ++h) {
     const int wh = __builtin_popcount(h);
     if (wh > 4) continue;
-    std::vector<Item> items;
-    for (uint32_t m = 0; m < nmid; ++m)
-      for (uint32_t l = 0; l < nlow; ++l) {
-        const int W = wh + __builtin_popcount(m) + __builtin_popcount(l);
-        const uint32_t key = (h << tb) | (m << (lb + RB)) | l;
-        if (W <= 4) items.push_back({W, key});
-        if (W <= (df ? 2 : 1))
-          for (uint32_t lo = 0; lo < (1u << RB); ++lo)
-            if (mask_kind(W, lo) == kM2 || mask_kind(W, lo) == kM2Top) items.push_back({kM2Rec, key | (lo << lb)});
-      }
-    auto rank = [](int type) { return type == kM2Rec ? 5 : 4 - type; };
-    std::stable_sort(items.begin(), items.end(), [&](const Item& a, const Item& b) { return rank(a.type) < rank(b.type); });
-    size_t k = 0;
-    while (k < items.size()) {
+    size_t k = pool.size();
+    for (int W = 4; W >= wh; --W)
+      for (uint32_t f : by[W - wh]) pool.push_back({W, (h << tb) | f});
+    if (wh <= most2)
+      for (uint32_t f : upto[most2 - wh])
+        for (uint32_t lo = 0; lo < (1u << RB); ++lo) {
+          const int kind = mask_kind(wh + __builtin_popcount(f), lo);
+          if (kind == kM2 || kind == kM2Top) pool.push_back({kM2Rec, (h << tb) | f | (lo << lb)});
+        }
+    while (k < pool.size()) {
       Chunk c;
       c.h = h;
+      c.first = k;
       int bytes = 16;
-      while (k < items.size()) {
-        const int type = items[k].type, need = 16 + bytes_of(type);
+      while (k < pool.size()) {
+        const int type = pool[k].type, need = 16 + bytes_of(type);
         if (bytes + need > auxb || c.count[type] == 255) break;
         bytes += need;
-        c.items.push_back(items[k]);
+        c.n++;
         c.count[type]++;
         c.cost += cost_of(type);
         ++k;
       }
-      if (c.items.empty()) throw std::runtime_error("row-block layout: a coset exceeds the chunk size");
-      all.push_back(std::move(c));
+      if (c.n == 0) throw std::runtime_error("row-block layout: a coset exceeds the chunk size");
+      all.push_back(c);
     }
   }
   // deal the chunks to the cs CTAs of a tile: the costliest first, each to the least loaded
@@ -842,6 +869,13 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, bool df
     lists[k].push_back(&c);
     load[k] += std::max(c.cost, fill);
   }
+  size_t total = 0;
+  for (const Chunk& c : all) {
+    total += 16;
+    for (size_t e = 0; e < c.n; ++e) total += 16 + size_t(bytes_of(pool[c.first + e].type));
+  }
+  out->blob.reserve(total + all.size() * sizeof(int4));
+  out->chunks.reserve(all.size());
   for (int k = 0; k < cs; ++k) {
     out->begin[k] = int(out->chunks.size());
     // spread the chunks whose copy takes longer than their arithmetic evenly among the others
@@ -852,23 +886,24 @@ int block_layout_T(const syk_terms* t, int lb, int mb, int cs, int auxb, bool df
       const bool small = i == nh || (j < nl && j * nh < i * nl);
       const Chunk& c = small ? *lists[k][nh + j++] : *lists[k][i++];
       const size_t b0 = out->blob.size();
-      out->blob.resize(b0 + 16 + 16 * c.items.size());
+      out->blob.resize(b0 + 16 + 16 * c.n);
       const uint4 head = make_uint4(uint32_t(c.count[4]) | uint32_t(c.count[3]) << 8 | uint32_t(c.count[2]) << 16 |
                                         uint32_t(c.count[1]) << 24,
                                     uint32_t(c.count[0]) | uint32_t(c.count[kM2Rec]) << 8, 0u, 0u);
       std::memcpy(out->blob.data() + b0, &head, 16);
-      for (size_t e = 0; e < c.items.size(); ++e) {
-        const uint32_t key = c.items[e].key;
+      for (size_t e = 0; e < c.n; ++e) {
+        const Item& item = pool[c.first + e];
+        const uint32_t key = item.key;
         const uint32_t low = key & (nlow - 1u), mid = (key >> (lb + RB)) & (nmid - 1u), lo = (key >> lb) & ((1u << RB) - 1u);
         uint4 rec = make_uint4(mid | (low << 16), 0u, 0u, uint32_t(out->blob.size() - b0));
-        if (c.items[e].type == kM2Rec) {
+        if (item.type == kM2Rec) {
           const int m = find_mask(t->m2_rec, t->n2, key);
           rec.x |= lo << 24;
           rec.y = t->m2_rec[4 * size_t(m) + 1];
           rec.z = t->m2_rec[4 * size_t(m) + 2];
           block_m2<RB>(t, lb, ng, m, df, &out->blob);
         } else {
-          const int W = c.items[e].type;
+          const int W = item.type;
           rec.x |= uint32_t(__builtin_popcount(low) & 1) << 31;
           int below = 0;
           for (int s = 0; s < nb; ++s) {
@@ -924,12 +959,16 @@ int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, b
     SYK_TRY(block_layout_host(t, rb, lb, mb, cs, auxb, df, &H));
     BlockLayout L;
     std::memcpy(L.begin, H.begin, sizeof(L.begin));
-    SYK_TRY(upload(&L.chunks, H.chunks.data(), H.chunks.size() * sizeof(int4)));
+    // one allocation and one copy: the chunk list behind the tables (a multiple of 16 bytes)
+    const size_t at = H.blob.size();
+    H.blob.resize(at + H.chunks.size() * sizeof(int4));
+    std::memcpy(H.blob.data() + at, H.chunks.data(), H.chunks.size() * sizeof(int4));
     const int rc = upload(&L.blob, H.blob.data(), H.blob.size());
     if (rc != SYK_OK) {
-      cudaFree(L.chunks);
+      cudaFree(L.blob);
       return rc;
     }
+    L.chunks = reinterpret_cast<int4*>(L.blob + at);
     it = t->block_dev.emplace(key, L).first;
   }
   *out = &it->second;

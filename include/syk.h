@@ -240,8 +240,8 @@ int syk_correlator_G_imag(const syk_terms* terms, double beta, int i, const doub
  * states per CTA, N = 28 at 2, N = 30 for one-state items; items split over
  * several CTAs only when the batch's split sub-items fill at least half the
  * SMs): each CTA takes sub-items from a device-side queue and evaluates their
- * entire chain -- Lanczos evolutions with FP64 scalars, tridiagonal
- * eigendecompositions, step control, Majoranas, dots -- with no host round
+ * entire chain -- Lanczos evolutions with FP64 scalars, exponentials of the
+ * tridiagonal projection, step control, Majoranas, dots -- with no host round
  * trip (syk_batch_persistent(0) turns this off).  The other items are taken,
  * largest first, by `nworkers` host threads, each with its own CUDA stream,
  * concurrently with that launch; every distinct (N, nstates) of theirs is
@@ -279,7 +279,7 @@ int syk_batch_plan(int N, int64_t nstates, int krylov_dim, int smem_limit, int* 
  * n <= 12 words): items in the persistent launch, items on the per-item path,
  * CTAs of the persistent launch; summed over its sub-items (one CTA's share of
  * an item's states): SM clock cycles spent in matvecs, in convergence checks
- * (tridiagonal eigendecompositions and step selection), in the combination
+ * (exponential of the tridiagonal projection and step selection), in the combination
  * coefficients of accepted bases (with their full eigendecomposition when no
  * check computed it) and in whole sub-items; H applications (states x
  * matvecs), convergence checks, separate full eigendecompositions; the

@@ -2,8 +2,8 @@
 // kernel launch over many small-sector work items.  Each CTA takes items from a device-side
 // queue (an atomic counter) and evaluates an item's whole regularized-OTOC chain (Eq. F_reg
 // by Eq. q_typicality, the chain of syk_otoc) by itself: every Krylov evolution (Supp. Sec.
-// I.B: Lanczos with the three-term recurrence, FP64 scalars, FP64 tridiagonal
-// eigendecompositions, Saad's error estimate and the step control of syk_expmv), the
+// I.B: Lanczos with the three-term recurrence, FP64 scalars, the FP64 exponential of the
+// projection (syk_check.cuh), Saad's error estimate and the step control of syk_expmv), the
 // Majorana applications and the final dots.  A work item is a sub-item: some of a coupling
 // draw's states (all of them, or a share of 2 or more when D x states would not fit), whose
 // sector vector fits in shared memory, so every matvec gathers its partner rows psi[x ^ m]
@@ -505,7 +505,7 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
           }
           cta_sum_cols<B>(p, S.red, S.n2);
         }
-        // alpha_j, beta_j (breakdown: beta_j = 0), sc_{j+1} = 1/beta_j, as k_lanczos_scalars
+        // alpha_j, beta_j (breakdown: beta_j = 0), sc_{j+1} = 1/beta_j, as k_update's last block
         if (tid < B) {
           const int c = tid;
           const double al = S.h[c].x;

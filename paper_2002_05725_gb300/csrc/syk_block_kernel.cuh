@@ -1,5 +1,6 @@
-// K1 variant: y = H psi in one parity sector (Supp. Sec. I.B) for complex64, with the rows of a
-// thread taken as a block of 2^RB consecutive compact indices (syk_block.cuh).
+// K1 variant: y = H psi in one parity sector (Supp. Sec. I.B), with the rows of a thread taken as a
+// block of 2^RB rows (syk_block.cuh): complex64 (BlockF32), complex128 in double-float arithmetic
+// (BlockDf, 8 rows; its figures stand in syk_block_df.cuh).  What follows is for complex64.
 //
 // A CTA owns a tile of 2^(LB+RB+MB) rows of all B states; thread t = (mid, low, state) owns the
 // 2^RB rows between its low and middle bits, for one state.  Per tile flip h the partner tile

@@ -1,6 +1,6 @@
 // Krylov expmv (Supp. Sec. I.B): Lanczos basis with full classical Gram-Schmidt
-// reorthogonalisation (two passes for complex128, one for complex64) (K2 + K7), eigendecomposition of the FP64
-// tridiagonal projection and its exponential (K3), and the combination
+// reorthogonalisation (two passes for complex128, one for complex64) (K2 + K7), the exponential
+// of the FP64 tridiagonal projection (K3: syk_check.cuh), and the combination
 // psi_out = V c (K4).  All scalars are FP64; complex64 vectors use FP32
 // arithmetic with FP64 accumulation of every reduction.
 //

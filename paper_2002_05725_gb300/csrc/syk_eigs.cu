@@ -44,7 +44,8 @@ bool tridiag_eig_lastrow(int m, std::vector<double>& d, std::vector<double>& e, 
     const double mu = d[q] - ee * ee / (dd + std::copysign(std::hypot(dd, ee), dd));
     double x = d[l] - mu, y = e[l];
     for (int k = l; k < q; ++k) {
-      const double r = std::hypot(x, y);
+      const double rr = x * x + y * y;  // hypot only where this leaves the range: it takes half the time
+      const double r = rr > 1e-280 && rr < 1e280 ? std::sqrt(rr) : std::hypot(x, y);
       const double c = r > 0.0 ? x / r : 1.0, s = r > 0.0 ? y / r : 0.0;
       if (k > l) e[k - 1] = r;
       const double a = d[k], b = e[k], cc = d[k + 1];
@@ -102,9 +103,23 @@ extern "C" int syk_lowest_eigenvalues(const syk_terms* terms, int parity, int dt
   int hstat[4] = {0, 0, 0, 0};
   int j0 = 0, mm = 0;
   bool converged = false, invariant = false;
+  // The check is a serial QR on the host, O(m^2) rotations (10 ms at m = 600), and outgrows the 16
+  // steps between two of them on the device (about 5 ms at D = 2^13): N = 28, 20 levels, 608 steps
+  // took 389 ms with one after the other, 307 now.  So the next steps are enqueued before the
+  // check, unless its worst residual bound, extrapolated from the last two checks, meets the
+  // tolerance: these steps would be wasted.  What a check sees does not depend on it.
+  int ahead = 0;                      // steps enqueued so far
+  double worst = -1.0, before = -1.0;  // worst bound relative to tol |T| of the last two checks; -1: none
+  struct Drain {  // steps in flight end before their workspace is given back
+    cudaStream_t st;
+    ~Drain() { cudaStreamSynchronize(st); }
+  } drain{st};
   while (j0 < m && !converged) {
     const int j1 = std::min(m, j0 + kCheck);
-    SYK_TRY(lanczos_steps(P, dtype, ws, j0, j1, st));
+    if (ahead < j1) {
+      SYK_TRY(lanczos_steps(P, dtype, ws, j0, j1, st));
+      ahead = j1;
+    }
     SYK_CUDA_CHECK(cudaMemcpyAsync(ha.data(), ws.alpha, sizeof(double) * j1, cudaMemcpyDeviceToHost, st));
     SYK_CUDA_CHECK(cudaMemcpyAsync(hb.data(), ws.beta, sizeof(double) * j1, cudaMemcpyDeviceToHost, st));
     SYK_CUDA_CHECK(cudaMemcpyAsync(hstat, ws.status, sizeof(int) * 2, cudaMemcpyDeviceToHost, st));
@@ -126,6 +141,10 @@ extern "C" int syk_lowest_eigenvalues(const syk_terms* terms, int parity, int dt
         invariant = true;
         break;
       }
+    if (!invariant && j1 < m && before >= 0.0 && worst * worst > before) {
+      ahead = std::min(m, j1 + kCheck);
+      SYK_TRY(lanczos_steps(P, dtype, ws, j1, ahead, st));
+    }
     d.assign(ha.begin(), ha.begin() + mm);
     e.assign(hb.begin(), hb.begin() + mm);  // e[mm-1] (the last beta) is unused by the solver
     if (!tridiag_eig_lastrow(mm, d, e, last)) {
@@ -144,6 +163,8 @@ extern "C" int syk_lowest_eigenvalues(const syk_terms* terms, int parity, int dt
     const double gap = 10.0 * tol * scale;
     int kk = 0;
     converged = true;
+    before = worst;
+    worst = 0.0;
     for (int i = 0; i < mm && kk < k; ++i) {
       const double th = d[ord[i]];
       if (kk > 0 && th - evals[kk - 1] <= gap) continue;
@@ -151,9 +172,13 @@ extern "C" int syk_lowest_eigenvalues(const syk_terms* terms, int parity, int dt
       const double r = beta_last * std::fabs(last[ord[i]]);
       if (resid) resid[kk] = r;
       if (!(r <= tol * scale)) converged = false;
+      worst = std::max(worst, r / (tol * scale));
       ++kk;
     }
-    if (kk < k) converged = false;
+    if (kk < k) {
+      converged = false;
+      worst = -1.0;
+    }
     if (invariant) break;
     j0 = j1;
   }

@@ -78,3 +78,20 @@ def test_lowest_eigenvalues_unconverged_bounds(torch):
     ev, res, n = syk.syk_lowest_eigenvalues(terms, 6, start, max_steps=16, tol=1e-12, check=False)
     ref = _distinct(np.linalg.eigvalsh(hm.H_sector_sparse(N, J, 0).toarray()))[:6]
     assert n == 16 and np.all(ev >= ref - 1e-12) and res.max() > 1e-12
+
+
+@pytest.mark.parametrize("N,k", [(16, 3), (18, 8), (22, 8)])
+def test_steps_enqueued_ahead_change_nothing(torch, N, k):
+    """Steps may be on the device before the check in front of them is done.  A run bounded to the
+    n steps it needs (none ahead of the last check) gives the same levels, up to the rounding of T
+    (n eps |T|, < 1e-12); one check fewer does not converge; nothing is in flight on return."""
+    terms = syk.syk_build_terms(N, inputs.couplings(N, 2))
+    start = inputs.random_states(N, 1, 3)[0]
+    ev, _, n = syk.syk_lowest_eigenvalues(terms, k, start, tol=1e-10)
+    assert torch.cuda.current_stream().query()
+    ev2, _, n2 = syk.syk_lowest_eigenvalues(terms, k, start, tol=1e-10, max_steps=n)
+    assert n2 == n and np.abs(ev - ev2).max() < 1e-12
+    if n % 16 == 0 and n - 16 >= k:
+        with pytest.raises(syk.SykError):
+            syk.syk_lowest_eigenvalues(terms, k, start, tol=1e-10, max_steps=n - 16)
+        assert torch.cuda.current_stream().query()

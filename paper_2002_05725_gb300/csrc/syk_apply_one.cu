@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(1 << NTB) k_apply_one(ApplyParams p, const int
   int g = 0;
   for (; g < nmine; ++g) {
     if (g + 1 < nmine) issue(g + 1);
-    const bool ok = tma::wait_bounded(&bar[g & 1], (g >> 1) & 1, tma::kWaitPolls);
+    const bool ok = tma::wait_bounded(&bar[g & 1], (g >> 1) & 1, tma::wait_polls());
     const int4 gr = __ldg(&groups[(int)crank + g * (int)csize]);
     const unsigned char* tb = sm + (g & 1) * BUFB;
     if (ok) {

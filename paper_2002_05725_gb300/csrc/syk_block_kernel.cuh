@@ -188,7 +188,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int st = q % kStages;
     // the refill's chunk is read ahead: the refill itself then starts at once
     const int4 refill = q + kStages < nq ? __ldg(&chunks[q0 + q + kStages]) : make_int4(0, 0, 0, 0);
-    if (!tma::wait_bounded(&full[st], (q / kStages) & 1, tma::kWaitPolls)) break;
+    // the lanes of a warp go on or give up together: a lane that left the loop alone would keep the
+    // others from ever passing the warp barriers below
+    if (!__all_sync(0xffffffffu, tma::wait_bounded(&full[st], (q / kStages) & 1, tma::wait_polls()))) break;
     const unsigned char* tb = sm + st * stageb;
     const unsigned char* cb = tb + tileb;
     const uint4 head = *reinterpret_cast<const uint4*>(cb);

@@ -58,12 +58,13 @@ __device__ __forceinline__ bool wait_bounded(uint64_t* b, uint32_t parity, uint3
   return false;
 }
 // Poll budget of the main-loop waits for staged tiles (a build-time knob: a build with 0 makes
-// every such wait give up at once, which exercises the timeout path), and of the drain that
+// every such wait give up at once, which exercises the timeout path; it may be an expression of
+// threadIdx, so that threads give up apart from one another), and of the drain that
 // lets in-flight copies land before a CTA that gave up exits (always the full budget).
 #ifndef SYK_WAIT_POLLS
 #define SYK_WAIT_POLLS (1u << 22)
 #endif
-constexpr uint32_t kWaitPolls = SYK_WAIT_POLLS;
+__device__ __forceinline__ uint32_t wait_polls() { return SYK_WAIT_POLLS; }
 constexpr uint32_t kDrainPolls = 1u << 22;
 // thread-block cluster helpers
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     if ((tid & 31) == 0) {
       __threadfence_block();
       if (atomicAdd(&done[st], 1) == nwarps - 1) {
+        __threadfence_block();  // the other warps' reads come before the refill's writes
         done[st] = 0;
         if (q + kStages < nq) issue(q + kStages, refill);
       }

@@ -165,19 +165,24 @@ __device__ inline double estimate(const Proj& p, double beta_last, double2 y0, d
   return beta_last * sqrt(num / den);
 }
 
-// sum_{k <= K} (2 - delta) I_k(w) e^{-w'} x[k] of the calling lane's own w (backward recurrence
-// and sum in one pass)
+// sum_{k <= K} (2 - delta) I_k(w) e^{-w'} x[k] of the calling lane's own w, in one pass: K serves
+// the lane of the largest w, and every lane's recurrence starts at the terms of its own w (the ones
+// above are below 1e-17).  Started at K, a small w would carry it beyond the range of a double (for
+// |w| = 4 and the terms of 128 to 1e210, squared in the division).
 __device__ inline double2 lane_sum(double2 w, int K, const double* x) {
   const bool neg = w.x < 0.0;
   const double2 v = neg ? make_double2(-w.x, -w.y) : w;
-  if (fma(v.x, v.x, v.y * v.y) < 1e-16) {
+  const double n2 = fma(v.x, v.x, v.y * v.y);
+  if (n2 < 1e-16) {
     const double f = neg ? -x[1] : x[1];
     return make_double2(x[0] + v.x * (f - x[0]), v.y * (f - x[0]));
   }
   const double2 iv = cdiv(make_double2(2.0, 0.0), v);
-  double2 hi = make_double2(0.0, 0.0), a = make_double2(1e-100, 0.0), sum = make_double2(0.0, 0.0);
+  double2 hi = make_double2(0.0, 0.0), a = make_double2(0.0, 0.0), sum = make_double2(0.0, 0.0);
   double2 dot = make_double2(0.0, 0.0);
+  const int start = min(K, terms(sqrt(n2))) + 4;
   for (int k = K + 4; k > 0; --k) {
+    if (k == start) a.x = 1e-100;
     sum.x += a.x;
     sum.y += a.y;
     if (k <= K) {
@@ -210,7 +215,7 @@ __device__ inline double select(const Proj& p, double beta_last, double s_top, d
     // |y|^2 = entry 0 of e^{2 s Re z T}; 1 in real time
     double den = 1.0;
     if (zr != 0.0) den = lane_sum(make_double2(2.0 * w.x, 0.0), terms(2.0 * fabs(zr) * hi * p.r), first).x;
-    const bool ok = !(den > 0.0) || beta_last * sqrt(fma(y.x, y.x, y.y * y.y) / den) <= tol;
+    const bool ok = den > 0.0 && beta_last * sqrt(fma(y.x, y.x, y.y * y.y) / den) <= tol;
     // the first step that fails bounds the bracket from above, the one before it from below
     const unsigned bad = ~__ballot_sync(0xffffffffu, ok && l < 31);
     const int f = __ffs(bad) - 1;

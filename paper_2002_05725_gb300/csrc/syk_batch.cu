@@ -575,7 +575,7 @@ __device__ __noinline__ void cta_expmv(const PArgs& a, const PItem& it, int sect
       __syncthreads();
       if (tid == 0) S.ctl->miss = 0;
       __syncthreads();
-      if (wp < B && !coefs_core(m_eff, B, wp, S.alpha, S.beta, S.beta0, zr, zi, s_acc,
+      if (wp < B && !coefs_core(m_eff, B, wp, S.alpha, S.beta, S.beta0, zr, zi, s_acc, tol,
                                 reinterpret_cast<double*>(S.A) + (size_t)wp * 4 * (cap + 1), S.cc, cap) && lane == 0)
         S.ctl->miss = 1;
       __syncthreads();

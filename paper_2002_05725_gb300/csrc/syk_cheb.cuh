@@ -8,7 +8,10 @@
 // modified Bessel functions, computed for all k at once by Miller's backward recurrence
 // I_{k-1} = I_{k+1} + (2k/w) I_k normalised with e^w = I_0 + 2 sum I_k (Olver et al., NIST
 // Handbook, 3.6 and 10.35; Re w < 0 by I_k(-w) = (-1)^k I_k(w)).  About |w| + 10 |w|^{1/3} + 15
-// terms reach 1e-17.  Everything stays relative to e^{|Re w|}, which cancels in Saad's estimate.
+// terms reach 1e-17.  Everything stays relative to e^{|Re w|}, which cancels in Saad's estimate;
+// the sums' rounding error, about 1e-16 on that scale, does not.  In imaginary time |y| may be far
+// below 1 there (Gershgorin's interval is wider than the spectrum, and e_1 has little weight at its
+// end), and the error is 1e-16/|y| of y: keeps() says whether that is small enough.
 //
 // Bound by the latency of dependent FP64 operations (FP64 runs at 1/64 of the FP32 rate here).  The
 // implicit QR that gave the same quantities is a chain of about m^2 Givens rotations of them: a
@@ -155,10 +158,23 @@ __device__ inline void sum(const Proj& p, int Ky, int K, const double2* ck, doub
   __syncwarp();
 }
 
-// Saad's estimate beta_last |y_{m-1}| / |y| from the sums (see step_error).
-__device__ inline double estimate(const Proj& p, double beta_last, double2 y0, double2 y1) {
+// |y|^2 from the sums
+__device__ inline double norm2(double2 y0, double2 y1) {
+  return warp_sum(fma(y0.x, y0.x, y0.y * y0.y) + fma(y1.x, y1.x, y1.y * y1.y));
+}
+
+// Whether sums of norm^2 n2 give y to the accuracy asked for.  Their error is at most 2e-16 (bases
+// of real couplings, N = 6 to 16, |w| up to 85, against 40-digit arithmetic), so y's is below 1.3e-14
+// of |y| (the eigendecomposition's: 1e-15 to 4e-14) or 2e-3 tol, whichever is larger.  |y| only grows
+// on its scale towards smaller steps, so a step search below needs no check of its own.
+__device__ __forceinline__ bool keeps(double n2, double tol) {
+  const double least = fmin(1.0 / 64.0, 1e-13 / tol);
+  return n2 >= least * least;
+}
+
+// Saad's estimate beta_last |y_{m-1}| / |y| from the sums and their norm^2 (see step_error).
+__device__ inline double estimate(const Proj& p, double beta_last, double2 y0, double2 y1, double den) {
   if (beta_last == 0.0) return 0.0;
-  const double den = warp_sum(fma(y0.x, y0.x, y0.y * y0.y) + fma(y1.x, y1.x, y1.y * y1.y));
   const double2 e = (p.m - 1) & 1 ? y1 : y0;
   const double num = __shfl_sync(0xffffffffu, fma(e.x, e.x, e.y * e.y), (p.m - 1) >> 1);
   if (!(den > 0.0)) return 0.0;

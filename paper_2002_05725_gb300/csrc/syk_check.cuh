@@ -59,7 +59,8 @@ __device__ inline void put_coefs(const cheb::Proj& p, double s, double zr, doubl
 // accepts s_target and its coefficients go to c (*have); else, in the basis' last check, the largest
 // step that passes (0 in earlier checks, where only the whole step counts).  Returns the step; error
 // bits go to status[0].  smd: the warp's own scratch for `cap` terms of the expansion, 4 (cap + 1)
-// doubles (at least 4m); beyond cap the eigendecomposition.  narrow: relative width of the step search.
+// doubles (at least 4m); beyond cap, or where the expansion loses digits (cheb::keeps), the
+// eigendecomposition.  narrow: relative width of the step search.
 constexpr int kCheckDoubles = 4 * (cheb::kMaxTerms + 1);
 static_assert(kCheckDoubles >= 4 * SYK_MAX_KRYLOV, "scratch of the eigendecomposition's rows");
 static __device__ double check_core(int m, int B, int b, const double* alpha, const double* beta, const double* beta0,
@@ -80,12 +81,16 @@ static __device__ double check_core(int m, int B, int b, const double* alpha, co
     cheb::coefs(w, K, ck);
     double2 y0, y1;
     cheb::sum(p, K, K2, ck, y0, y1, last ? first : nullptr, last ? lastv : nullptr);
-    if (cheb::estimate(p, bl, y0, y1) <= tol) {
-      put_coefs(p, s_target, zr, zi, y0, y1, beta0[b], B, b, c);
-      *have = true;
-      return s_target;
+    const double n2 = cheb::norm2(y0, y1);
+    if (cheb::keeps(n2, tol)) {
+      if (cheb::estimate(p, bl, y0, y1, n2) <= tol) {
+        put_coefs(p, s_target, zr, zi, y0, y1, beta0[b], B, b, c);
+        *have = true;
+        return s_target;
+      }
+      return last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv, narrow) : 0.0;
     }
-    return last ? cheb::select(p, bl, s_target, tol, zr, zi, first, lastv, narrow) : 0.0;
+    __syncwarp();  // the terms have been read: their memory becomes the decomposition's
   }
   double *d, *q0, *qm;
   const bool ok = eig_column<false>(m, B, b, alpha, beta, smd, &d, &q0, &qm);
@@ -95,9 +100,10 @@ static __device__ double check_core(int m, int B, int b, const double* alpha, co
 }
 
 // The coefficients of column b at the step s by one warp (put_coefs), false when they need more than
-// `cap` terms; smd: 2 (cap + 1) doubles.
+// `cap` terms or the expansion loses digits (cheb::keeps); smd: 2 (cap + 1) doubles.
 static __device__ bool coefs_core(int m, int B, int b, const double* alpha, const double* beta, const double* beta0,
-                                  double zr, double zi, double s, double* smd, double2* c, int cap = cheb::kMaxTerms) {
+                                  double zr, double zi, double s, double tol, double* smd, double2* c,
+                                  int cap = cheb::kMaxTerms) {
   const cheb::Proj p = cheb::load(m, alpha + b, beta + b, B);
   const double2 w = make_double2(s * zr * p.r, s * zi * p.r);
   const double aw = sqrt(fma(w.x, w.x, w.y * w.y));
@@ -107,6 +113,7 @@ static __device__ bool coefs_core(int m, int B, int b, const double* alpha, cons
   cheb::coefs(w, K, ck);
   double2 y0, y1;
   cheb::sum(p, K, K, ck, y0, y1, nullptr, nullptr);
+  if (!cheb::keeps(cheb::norm2(y0, y1), tol)) return false;
   put_coefs(p, s, zr, zi, y0, y1, beta0[b], B, b, c);
   return true;
 }

@@ -443,10 +443,12 @@ inline size_t check_smem() { return kCheckDoubles * sizeof(double); }
 
 // c[k*B + b] = beta0_b (e^{s z T_b} e_1)_k, one warp per column.
 __device__ void coef_column(int m, int B, const double* __restrict__ alpha, const double* __restrict__ beta,
-                            const double* __restrict__ beta0, double zr, double zi, double s, int* status, double2* c) {
+                            const double* __restrict__ beta0, double zr, double zi, double s, double tol, int* status,
+                            double2* c) {
   extern __shared__ __align__(16) double smd[];
   const int b = blockIdx.x;
-  if (coefs_core(m, B, b, alpha, beta, beta0, zr, zi, s, smd, c)) return;
+  if (coefs_core(m, B, b, alpha, beta, beta0, zr, zi, s, tol, smd, c)) return;
+  __syncwarp();  // the terms have been read: their memory becomes the decomposition's
   double *d, *q0, *qm;
   if (!eig_column<true>(m, B, b, alpha, beta, smd, &d, &q0, &qm) && threadIdx.x == 0) atomicOr(status, 2);
   for (int k = threadIdx.x; k < m; k += 32) {
@@ -468,8 +470,9 @@ struct Steps {
 };
 __global__ void __launch_bounds__(32) k_krylov_coefs(int m, int B, const double* __restrict__ alpha,
                                                      const double* __restrict__ beta, const double* __restrict__ beta0,
-                                                     double zr, double zi, Steps st, int* status, double2* c, size_t cs) {
-  coef_column(m, B, alpha, beta, beta0, zr, zi, st.s[blockIdx.y], status, c + blockIdx.y * cs);
+                                                     double zr, double zi, Steps st, double tol, int* status, double2* c,
+                                                     size_t cs) {
+  coef_column(m, B, alpha, beta, beta0, zr, zi, st.s[blockIdx.y], tol, status, c + blockIdx.y * cs);
 }
 
 inline size_t coef_smem(int m) {
@@ -568,7 +571,7 @@ __global__ void __launch_bounds__(32) k_krylov_coefs_dev(int B, const double* __
                                                          const double* __restrict__ beta, const double* __restrict__ beta0,
                                                          const ExpJob* __restrict__ job, const DevCtl* __restrict__ ctl,
                                                          int* status, double2* c) {
-  coef_column(ctl->m_eff, B, alpha, beta, beta0, job->zr, job->zi, ctl->ds, status, c);
+  coef_column(ctl->m_eff, B, alpha, beta, beta0, job->zr, job->zi, ctl->ds, job->tol, status, c);
 }
 
 // After the check that ends Lanczos segment [.., j1): converged when the accepted step covers
@@ -1080,7 +1083,7 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
         ++n;
       }
       double2* cq = reinterpret_cast<double2*>(ws.Q);
-      k_krylov_coefs<<<dim3(int(B), n), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp,
+      k_krylov_coefs<<<dim3(int(B), n), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp, tol,
                                                                     ws.status, cq, cset);
       count_launch();
       Ops<R>::combine(ws, m_eff, nullptr, cq, cset, outs + next, n, st);
@@ -1094,7 +1097,7 @@ int expmv_T(const ApplyParams& P_in, int dtype, std::complex<double> z, const vo
     if (!final_basis) {  // restart from the state at the end of this basis' step
       Steps sp = {};
       sp.s[0] = s_acc;
-      k_krylov_coefs<<<dim3(int(B), 1), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp,
+      k_krylov_coefs<<<dim3(int(B), 1), 32, coef_smem(m_eff), st>>>(m_eff, int(B), ws.alpha, ws.beta, ws.beta0, zr, zi, sp, tol,
                                                                     ws.status, ws.c, 0);
       count_launch();
       Ops<R>::combine(ws, m_eff, nullptr, ws.c, 0, outs + nf - 1, 1, st);

@@ -53,3 +53,16 @@ def test_step_search_c128(N, m, z):
 @pytest.mark.parametrize("m,z", [(6, -110.0), (6, 110.0), (8, -105.0), (8, 105.0), (12, -110.0)])
 def test_step_search_c64(N, m, z):
     _check(N, complex(z), m, "c64")
+
+
+@pytest.mark.parametrize("N", [6, 8, 10, 12])
+@pytest.mark.parametrize("reach", [-60.0, -40.0, -20.0, 20.0, 40.0, 60.0, -30.0 + 20.0j, 45.0 + 10.0j])
+def test_invariant_basis(N, reach):
+    """Bases that span the sector (estimate 0: whatever the expansion gives is accepted), with
+    |Re z| (half the spectrum's width) of `reach`: the result is far below the scale of the sums."""
+    J = inputs.couplings(N, 21)
+    for sector in (0, 1):
+        E = np.linalg.eigvalsh(hm.H_sector_sparse(N, J, sector).toarray())
+        z = reach / (0.5 * (E[-1] - E[0]))
+        _check(N, complex(z), 40, "c128", sector=sector)
+        _check(N, complex(z), 40, "c64", sector=sector)

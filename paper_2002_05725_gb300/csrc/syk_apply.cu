@@ -238,12 +238,15 @@ int launch_epilogue(const ApplyParams& p, void* y, int64_t batch, cudaStream_t s
   return SYK_OK;
 }
 
-// The row-block kernel (complex64; complex128 takes the split copy): the tuned shape (variant 4 or 5), or its launch rule where nothing
-// is tuned; returns 1 if it does not apply.
+// The row-block kernel (complex64; complex128 takes the split copy): the tuned shape (variant 4 or
+// 5), or its launch rule where nothing is tuned or the tuned shape does not fit; returns false if
+// it does not apply.
 bool block_choice(const ApplyParams& p, int dtype, int64_t batch, BlockShape* sh) {
   TileChoice tc;
-  if (tile_choice_lookup(p.n * 2, dtype, batch, &tc))
-    return tc.var >= kBlockVariant && block_shape(p.n, batch, dtype, block_rows(tc.var), tc.ntb - 4, tc.cs, sh);
+  if (tile_choice_lookup(p.n * 2, dtype, batch, &tc)) {
+    if (tc.var < kBlockVariant) return false;
+    if (block_shape(p.n, batch, dtype, block_rows(tc.var), tc.ntb - 4, tc.cs, sh)) return true;
+  }
   return block_default(p.n, batch, dtype, sh);
 }
 int try_block(const ApplyParams& p, int dtype, const void* psi, void* y, int64_t batch, cudaStream_t st) {

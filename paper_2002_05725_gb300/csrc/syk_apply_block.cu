@@ -34,7 +34,9 @@ bool block_shape(int n, int64_t batch, int dtype, int rb, int mb, int cs, BlockS
   const bool df = dtype == SYK_C128;
   if (batch < 1 || batch > 32 || mb < 0 || (rb != 3 && rb != 5) || (df && (rb != 3 || !pow2(batch) || batch > 16))) return false;
   *sh = {rb, low_bits(batch), mb, cs, block_aux(n, rb, df), df};
-  return sh->lb + rb + mb <= n - 1 && (batch << (sh->lb + mb)) <= 256 &&
+  const int tb = sh->lb + rb + mb;
+  const int64_t D = int64_t(1) << (n - 1);
+  return tb <= n - 1 && (batch << (sh->lb + mb)) <= 256 && (D >> tb) * cs <= ep_capacity(D) &&
          block_smem(batch, sh->lb, rb, mb, sh->auxb, df ? 16 : 8) <= kMaxSmemPerCta;
 }
 

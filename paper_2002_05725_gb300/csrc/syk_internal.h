@@ -98,6 +98,7 @@ struct ApplyParams {
   int* ep_nblk;
   int64_t ep_cap;          // host-side: capacity of ep_part in CTAs
 };
+int64_t ep_capacity(int64_t D);  // of a Krylov workspace for vectors of dimension D
 
 // Chunks of X-masks sharing the compact-mask bits h above a tile of 2^tb rows, at
 // most gmax popcount-4 masks per chunk: {h | first-chunk-of-h << 31, first
@@ -172,7 +173,8 @@ struct BlockShape {
 };
 int block_aux(int n, int rb, bool df);  // the smallest auxb
 size_t block_smem(int64_t B, int lb, int rb, int mb, int auxb, int elem);
-// The shape with 2^rb rows per thread (3 or 5), mb middle bits and cs CTAs per tile, if it exists.
+// The shape with 2^rb rows per thread (3 or 5), mb middle bits and cs CTAs per tile, if it exists
+// and its CTAs fit a Krylov workspace's epilogue buffer.
 bool block_shape(int n, int64_t batch, int dtype, int rb, int mb, int cs, BlockShape* sh);
 // The launch rule of the matvec (complex128: double-float); false: the sector is too small, or too many states.
 bool block_default(int n, int64_t batch, int dtype, BlockShape* sh);

@@ -727,11 +727,12 @@ int lanczos_step(const ApplyParams& P, int dtype, KrylovWS& ws, int j, int orth,
 
 size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
-// CTAs a matvec launch may have (its epilogue writes one partial per CTA and column): tiles of
-// at least 64 rows, clusters of at most 8; the row kernel's epilogue uses at most kRedBlocksCap.
-int64_t ep_capacity(int64_t D) { return std::max<int64_t>(D / 8, kRedBlocksCap); }
-
 }  // namespace
+
+// CTAs a matvec launch may have (its epilogue writes one partial per CTA and column): tiles of
+// at least 64 rows, clusters of at most 8 (smaller tiles, smaller clusters: block_shape); the row
+// kernel's epilogue uses at most kRedBlocksCap.
+int64_t ep_capacity(int64_t D) { return std::max<int64_t>(D / 8, kRedBlocksCap); }
 
 // by dtype code: complex64 defaults to the three-term recurrence (as accurate as full
 // Gram-Schmidt at FP32 rounding, measured against complex128 and the oracle, and 11 % less

@@ -345,8 +345,8 @@ int syk_autotune_apply(const syk_terms* terms, int parity, int dtype, int64_t ba
 /* syk_autotune_export / _import -- the tuned table as JSON
  * ({"apply_tiles": [{"N":..,"dtype":..,"batch":..,"ntb":..,"cluster":..,"variant":..,"ms":..}]};
  * variant 0 is the plain tiled kernel, 1..3 the complex64 coset kernel with 2^variant rows
- * per thread, 4 and 5 the row-block kernel with 32 (complex64) and 8 rows per thread (complex64,
- * and complex128 with up to 4 states); a missing variant reads as 0),
+ * per thread, 4 and 5 the row-block kernel with 32 (complex64) and 8 rows per thread (complex64
+ * and complex128); a missing variant reads as 0),
  * so a tuning run can be cached in a file and reloaded. */
 int syk_autotune_export(char* buf, size_t len);
 int syk_autotune_import(const char* json);

@@ -928,9 +928,10 @@ extern "C" int syk_autotune_import(const char* json) {
     if (num("N", &N) && num("dtype", &dt) && num("batch", &b) && num("ntb", &ntb) && num("cluster", &cs)) {
       num("ms", &ms);
       num("variant", &var);
-      const bool block = dt == SYK_C64 ? (var == kBlockVariant || var == kLastVariant) &&
-                                             (b == 1 || b == 2 || b == 4 || b == 8 || b == 16)
-                                       : dt == SYK_C128 && var == kLastVariant && (b == 1 || b == 2 || b == 4);
+      // (what syk_autotune_apply tries, and so may export)
+      const bool block = (dt == SYK_C64 ? var == kBlockVariant || var == kLastVariant
+                                        : dt == SYK_C128 && var == kLastVariant) &&
+                         (b == 1 || b == 2 || b == 4 || b == 8 || b == 16);
       if (ntb < 6 || ntb > 8 || (cs != 1 && cs != 2 && cs != 4 && cs != 8) ||
           !(block || coset_var_ok(int(dt), int64_t(b), int(var)))) {
         set_error("syk_autotune_import: invalid entry (ntb=%g cluster=%g variant=%g)", ntb, cs, var);

@@ -33,3 +33,27 @@ def test_expmv_with_every_shape(N, B):
                     assert rel(y, ref) < TOL["c64"], (var, ntb, cs)
     finally:
         syk.syk_autotune_reset()
+
+
+@pytest.mark.parametrize("B", [1, 2, 4, 8, 16])
+def test_complex128_shapes_vs_oracle(B):
+    """Every complex128 row-block shape that the table takes, against the FP64 oracle."""
+    from oracle import hamiltonian as hm
+    torch = torch_or_skip()
+    syk.load(build_if_missing=True)
+    N = 24
+    J = inputs.couplings(N, 6)
+    terms = syk.syk_build_terms(N, J)
+    H = hm.H_sector_sparse(N, J, 1)
+    psi = inputs.random_states(N, B, 4)
+    x = to_dev(torch, psi, "c128")
+    try:
+        for ntb in (6, 7, 8):
+            for cs in (1, 2, 4, 8):
+                syk.syk_autotune_reset()
+                syk.syk_autotune_import(json.dumps({"apply_tiles": [
+                    {"N": N, "dtype": 2, "batch": B, "ntb": ntb, "cluster": cs, "variant": 5}]}))
+                y = syk.syk_apply_H(terms, 1, x).cpu().numpy().reshape(-1, B)
+                assert rel(y, H @ psi.T) < TOL["c128"], (ntb, cs)
+    finally:
+        syk.syk_autotune_reset()

@@ -93,13 +93,16 @@ int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, voi
   a.nt = a.SE << sh.mb;
   a.auxb = sh.auxb;
   const BlockLayout* L = nullptr;
-  int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, false, &L);
+  int lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, false, false, &L);
   if (lr > 0 && !p.no_alloc) {
-    // the first launch of a shape builds its layout, which a stream under capture cannot
+    // The first launch of a shape builds its layout, under capture too: the kernels that would stand
+    // in have layouts of their own, which nothing builds any more where this kernel is the default.
+    // (The query fails on the legacy stream while another one is under capture: then the former
+    // kernels take over, as far as they can.)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
-    else if (cap == cudaStreamCaptureStatusNone)
-      lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, true, &L);
+    else
+      lr = block_layout(p.terms, sh.rb, sh.lb, sh.mb, sh.cs, sh.auxb, sh.df, true, cap != cudaStreamCaptureStatusNone, &L);
   }
   if (lr != SYK_OK) return lr > 0 ? 1 : lr;
   for (int k = 0; k < 9; ++k) a.begin[k] = L->begin[k];

@@ -162,7 +162,9 @@ struct BlockLayout {
   unsigned char* blob = nullptr;
   int begin[9] = {};
 };
-int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc,
+// may_alloc false: 1 if the layout is not built yet.  capturing: a stream is under capture by this
+// thread, whose allocations and copies would break it; the build then keeps out of its way.
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc, bool capturing,
                  const BlockLayout** out);
 
 // Shape of a row-block launch: rows per thread 2^rb, low and middle bits, CTAs per tile, bytes

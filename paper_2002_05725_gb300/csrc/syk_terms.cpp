@@ -946,7 +946,25 @@ int block_layout_host(const syk_terms* t, int rb, int lb, int mb, int cs, int au
   }
 }
 
-int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc,
+namespace {
+
+// upload() beside a stream under capture: the thread's allocations are allowed while its capture mode
+// is relaxed, and the copy runs on the thread's own stream (the legacy stream may not be used).
+int upload_beside_capture(unsigned char** dst, const void* src, size_t bytes) {
+  struct Relaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  } relaxed;
+  SYK_CUDA_CHECK(cudaMalloc(dst, bytes));
+  SYK_CUDA_CHECK(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, cudaStreamPerThread));
+  SYK_CUDA_CHECK(cudaStreamSynchronize(cudaStreamPerThread));
+  return SYK_OK;
+}
+
+}  // namespace
+
+int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, bool df, bool may_alloc, bool capturing,
                  const BlockLayout** out) {
   if (may_alloc) SYK_TRY(ensure_device_tables(t));
   std::lock_guard<std::mutex> lock(t->mtx);
@@ -963,7 +981,8 @@ int block_layout(const syk_terms* t, int rb, int lb, int mb, int cs, int auxb, b
     const size_t at = H.blob.size();
     H.blob.resize(at + H.chunks.size() * sizeof(int4));
     std::memcpy(H.blob.data() + at, H.chunks.data(), H.chunks.size() * sizeof(int4));
-    const int rc = upload(&L.blob, H.blob.data(), H.blob.size());
+    const int rc = capturing ? upload_beside_capture(&L.blob, H.blob.data(), H.blob.size())
+                             : upload(&L.blob, H.blob.data(), H.blob.size());
     if (rc != SYK_OK) {
       cudaFree(L.blob);
       return rc;

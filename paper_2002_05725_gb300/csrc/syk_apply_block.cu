@@ -70,12 +70,20 @@ bool block_default(int n, int64_t batch, int dtype, BlockShape* sh) {
   // states: 68 and 60; N = 38, 8 states: 2.9 and 1.9 ms).  Full tiles (256 threads, one CTA per
   // SM) halve the copies of 128-thread ones (N = 40, 16 states: 8.7 against 13.7 ms); a cluster
   // splits a tile's chunks while that leaves at most about one CTA per SM (N = 32, 16 states, 64
-  // tiles: 254 us with 2 CTAs a tile, 466 with 1, 263 with 4; N = 38, 8 states, 256 tiles: 1.93 ms
-  // with 1, 1.96 with 2).  Clusters of 8 only with small CTAs, several to an SM.
+  // tiles: 248 us with 2 CTAs a tile, 459 with 1; N = 38, 8 states, 256 tiles: 1.97 ms with 1, 2.01
+  // with 2).  Clusters of 8 only with small CTAs, several to an SM.
+  // 4, 8 and 16 states take more: each CTA of a cluster sums a share of the masks, and shorter FP32
+  // chains keep the rounding error below that of the coset kernel, whose clusters were of 4 or 8
+  // there.  Relative error (2-norm) of that one, with the rule above and with this one, and the time
+  // it takes: N = 32, 16 states 4.1e-7, 5.4e-7, 3.8e-7, 248 -> 258 us; N = 34, 8 states 4.6e-7, 6.1e-7,
+  // 4.3e-7, 320 -> 332 us; N = 36, 4 states 5.2e-7, 6.9e-7, 4.9e-7, 451 -> 474 us; N = 38, 4 states
+  // 8.3e-7, 1.1e-6, 7.7e-7, 1.08 -> 1.09 ms.  Where a tile has one CTA, launch_apply_block sums in parts.
   if (D * batch > (int64_t(1) << 16)) {
     const int64_t tiles = D >> std::min(n - 1, lb + 5 + full);
     const int mb = tiles >= 25 ? full : full - 1;
-    const int cs = tiles >= 100 ? 1 : tiles >= 50 ? 2 : 4;
+    int cs = tiles >= 100 ? 1 : tiles >= 50 ? 2 : 4;
+    if (cs == 2 && (batch == 4 || batch == 8 || batch == 16)) cs = 4;
+    if (cs == 1 && batch == 4 && tiles < 200) cs = 2;
     if (block_shape(n, batch, dtype, 5, mb, cs, sh)) return true;
   }
   for (int mb = std::min(3, full); mb >= 0; --mb)
@@ -109,6 +117,13 @@ int launch_apply_block(const ApplyParams& p, int64_t batch, const void* psi, voi
   const int which = a.SE != 16 ? kBlockAny : sh.lb == 0 ? kBlock16 : batch == 8 ? kBlockShare : kBlockPow2;
   const bool share = which == kBlock16 || which == kBlockShare;
   if (sh.df) return launch_block_df(p, a, sh.cs, L, psi, y, st);
+  // 8 and 16 states with one CTA a tile: in parts up to the size where the coset kernel still split a
+  // row over 4 CTAs or more (from N = 38, 16 states, and N = 40, 8 states, on one chain is no worse
+  // than it was: 1.11e-6 against 1.17e-6, 1.22e-6 against 1.30e-6)
+  if (sh.rb == 5 && share && sh.cs == 1 && p.D * batch < (int64_t(1) << 22)) {
+    a.part = (a.begin[1] + 7) / 8;
+    return launch_block32_parts(p, a, which, L, psi, y, st);
+  }
   if (sh.rb == 5)
     return share ? launch_block32_share(p, a, which, sh.cs, L, psi, y, st)
                  : launch_block32_direct(p, a, which, sh.cs, L, psi, y, st);

@@ -21,10 +21,11 @@
 // against 256 of the FP32 pipe) 20 % less.
 // Measured (GB300, per matvec, before -> after; before: the faster of the coset, tiled,
 // one-state and row kernels' defaults): N = 40, 16 states 10.45 -> 8.44 ms (40 TFLOP/s); N = 48,
-// 1 state 59.1 -> 19.1 ms; N = 36, 8 states 1.70 -> 0.78 ms; N = 34, 6 states 2.28 -> 0.39 ms;
-// N = 32, 16 states 408 -> 253 us; N = 28, 8 states 136 -> 42 us, 1 state 328 -> 27 us; N = 20, 8
-// states 69 -> 16 us.  Errors against 64-bit sums are 0.4 to 0.7 of the former kernels' (one
-// rounding per product-sum instead of two).
+// 1 state 59.1 -> 19.1 ms; N = 36, 8 states 1.70 -> 0.80 ms; N = 34, 6 states 2.28 -> 0.39 ms;
+// N = 32, 16 states 408 -> 258 us; N = 28, 8 states 136 -> 42 us, 1 state 328 -> 27 us; N = 20, 8
+// states 69 -> 16 us.  Errors against 64-bit sums are 0.5 to 0.95 of the former kernels' for 1, 2, 4,
+// 8 and 16 states, N = 20 to 42 (one rounding per product-sum instead of two, but longer chains: see
+// PARTS), and 0.25 to 0.65 of the row kernel's for other counts.
 // Tried and slower: 16 rows per thread with twice the threads (9.1 against 8.7 ms at N = 40, more
 // shared-memory reads per mask); coefficients stored ready-paired (wider reads cost the port more
 // than the register moves they save); two-spin coefficients per thread instead of per row block
@@ -46,6 +47,7 @@ struct BlockArgs {
   int SE;        // elements per row slot: B << LB
   int nt;        // threads that own rows: SE << MB
   int auxb;      // bytes of a stage for a chunk's records and tables
+  int part;      // PARTS: chunks after which the sums so far go to y
   int begin[9];  // chunk range of each CTA of a tile
 };
 
@@ -121,7 +123,14 @@ __device__ __forceinline__ T ld_cluster_elem(uint32_t a) {
 }
 
 // SEC: SE when known at compile time (16), so that row offsets are immediates; 0 otherwise.
-template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB>
+// PARTS: a row's sum is taken in eight parts, added up in y.  In one FP32 chain its rounding error grows
+// with the number of masks, and where the kernels before this one split a row over 4 or 8 CTAs of a
+// cluster, one chain was worse than they were (launch_apply_block says where that is).  Relative error
+// (2-norm) of the former kernels, of one chain and of the parts, and the time of the latter two:
+// N = 34, 16 states 4.6e-7, 8.6e-7, 3.6e-7, 595 -> 600 us; N = 36, 8 states 5.2e-7, 9.7e-7, 3.9e-7,
+// 786 -> 799 us; N = 36, 16 states 7.4e-7, 9.8e-7, 4.0e-7, 1.50 -> 1.52 ms (a part reads and writes the
+// CTA's 64 KB of y).  Four parts gave 5.0e-7, 5.4e-7, 5.6e-7: their chunks hold unequal numbers of masks.
+template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB, bool PARTS>
 __global__ void __launch_bounds__(MAXT, MINB)
     k_apply_block(ApplyParams p, const BlockArgs c, const int4* __restrict__ chunks, const unsigned char* __restrict__ blob,
                   const void* __restrict__ psi, typename Arith<RB, SHARE>::Out* __restrict__ y) {
@@ -184,7 +193,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
     for (int q = 0; q < kStages && q < nq; ++q) issue(q, __ldg(&chunks[q0 + q]));
 
   int q = 0;
-  for (; q < nq; ++q) {
+  for (int qe = PARTS ? min(c.part, nq) : nq;; qe = min(qe + c.part, nq)) {
+  for (; q < qe; ++q) {
     const int st = q % kStages;
     // the refill's chunk is read ahead: the refill itself then starts at once
     const int4 refill = q + kStages < nq ? __ldg(&chunks[q0 + q + kStages]) : make_int4(0, 0, 0, 0);
@@ -246,6 +256,21 @@ __global__ void __launch_bounds__(MAXT, MINB)
     }
     __syncwarp();
   }
+  if (!PARTS || q < qe || q == nq) break;  // (q < qe: a wait gave up)
+  if constexpr (PARTS) {  // (a thread's rows of y are its own)
+    if (active) {
+      Out* __restrict__ yt = y + (size_t)tile * (tileb / kElem) + (size_t)(mid << RB) * SE + el;
+      const bool first = q == c.part;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        Sum v = A::get(acc, r);
+        if (!first) A::add(v, yt[r * SE]);
+        yt[r * SE] = v;
+      }
+    }
+    A::zero(acc);
+  }
+  }
   if (q < nq) *lost = 1;
   __syncthreads();
   if (*lost) {
@@ -302,7 +327,12 @@ __global__ void __launch_bounds__(MAXT, MINB)
   } else {
     if (active) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) emit((size_t)((mid << RB) + r) * SE + el, A::get(acc, r), r);
+      for (int r = 0; r < R; ++r) {
+        const size_t e = (size_t)((mid << RB) + r) * SE + el;
+        Sum v = A::get(acc, r);
+        if (PARTS && nq > c.part) A::add(v, y[gbase + e]);
+        emit(e, v, r);
+      }
     }
     __syncthreads();
   }
@@ -328,12 +358,14 @@ __global__ void __launch_bounds__(MAXT, MINB)
 enum { kBlock16 = 0, kBlockShare = 1, kBlockPow2 = 2, kBlockAny = 3 };
 int launch_block32_share(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                          const void* psi, void* y, cudaStream_t st);
+int launch_block32_parts(const ApplyParams& p, const BlockArgs& a, int which, const BlockLayout* L, const void* psi, void* y,
+                         cudaStream_t st);
 int launch_block_df(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLayout* L, const void* psi, void* y,
                     cudaStream_t st);
 int launch_block32_direct(const ApplyParams& p, const BlockArgs& a, int which, int cs, const BlockLayout* L,
                           const void* psi, void* y, cudaStream_t st);
 
-template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB>
+template <template <int, bool> class Arith, int RB, int SEC, bool LOWB, bool SHARE, int MAXT, int MINB, bool PARTS = false>
 int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLayout* L, const void* psi, void* y,
              cudaStream_t st) {
   const int tb = a.LB + RB + a.MB;
@@ -344,7 +376,7 @@ int launch_block(const ApplyParams& p, const BlockArgs& a, int cs, const BlockLa
   }
   using Out = typename Arith<RB, SHARE>::Out;
   const size_t smem = block_smem(a.B, a.LB, RB, a.MB, a.auxb, Arith<RB, SHARE>::kElem);
-  const auto kern = k_apply_block<Arith, RB, SEC, LOWB, SHARE, MAXT, MINB>;
+  const auto kern = k_apply_block<Arith, RB, SEC, LOWB, SHARE, MAXT, MINB, PARTS>;
   SYK_TRY(ensure_smem_limit((const void*)kern, (int)kMaxSmemPerCta));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ntiles * cs), 1, 1);

@@ -95,11 +95,11 @@ def peaks():
 
 
 def matvec_kernel(tile, states, dtype):
-    """Name and source file of the matvec kernel a tuned launch shape selects."""
+    """Name and source files of the matvec kernel a tuned launch shape selects."""
     if tile and tile.get("variant", 0) >= 4:
         rows = 32 if tile["variant"] == 4 else 8
         return (f"k_apply_block<{rows} rows, {states} states, {1 << tile['ntb']} threads> (cluster {tile['cluster']})",
-                "block", "syk_block.cuh")
+                "block", "syk_block_kernel.cuh syk_block.cuh")
     if tile and tile.get("variant", 0) > 0:
         return (f"k_apply_coset<{states}, RB={tile['variant']}, ntb={tile['ntb']}> (cluster {tile['cluster']})",
                 "coset", "syk_apply_coset.cu")
@@ -113,10 +113,10 @@ def ncu_traffic(N, states, dtype, kind="tiled", source="syk_apply.cu"):
     or None if there is none or the kernel source changed since it was captured."""
     import hashlib
     path = os.path.join(ROOT, "profiles", f"apply_{kind}_N{N}_B{states}_{dtype}.md")
-    src = os.path.join(ROOT, "paper_2002_05725_gb300", "csrc", source)
+    csrc = os.path.join(ROOT, "paper_2002_05725_gb300", "csrc")
     try:
         text = open(path).read()
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()
+        sha = hashlib.sha256(b"".join(open(os.path.join(csrc, f), "rb").read() for f in source.split())).hexdigest()
     except OSError:
         return None, None
     vals = {}

@@ -374,8 +374,10 @@ int syk_counters(int64_t* h_applies, int64_t* krylov_bases, int64_t* launches, i
 
 /* syk_matvec_launches -- matvec launches since the last reset by kernel family (any
  * pointer may be NULL): the row kernel (small sectors, other batch sizes, unaligned
- * vectors), the tiled kernel and the complex64 coset kernels (row blocks among them).  A Lanczos segment replayed
- * from a captured graph adds the launches it recorded.  reset != 0 zeroes them. */
+ * vectors; the steps of a small sector's one-launch basis), the tiled kernels (the complex128
+ * row-block kernel among them) and the complex64 coset kernels (the complex64 row-block kernel
+ * among them).  A Lanczos segment replayed from a captured graph adds the launches it recorded.
+ * reset != 0 zeroes them. */
 int syk_matvec_launches(int64_t* rows, int64_t* tiled, int64_t* coset, int reset);
 
 /* syk_profile_enable / syk_profile_read -- CUDA-event timing of every apply_H
@@ -394,7 +396,9 @@ int syk_profile_enable(int on);
  * device (conditional WHILE and IF nodes): the chain is enqueued without host
  * synchronisation, with bit-identical results; the graph is built once per workspace, term
  * set and sector, which costs more than it saves for a chain run only once (syk_expmv and
- * the gradients stay host-driven).  Graphs are not used while profiling is enabled. */
+ * the gradients stay host-driven).  In small sectors (up to 2^14 nonzeros of H times states:
+ * N = 12 to 16 states, N = 14 to 4, N = 16 one) a Krylov basis is one launch with one host read
+ * in every mode.  Graphs are not used while profiling is enabled. */
 int syk_use_graphs(int on);
 int syk_profile_read(int64_t* launches, double* total_ms, int reset);
 

@@ -48,7 +48,10 @@ bool block_default(int n, int64_t batch, int dtype, BlockShape* sh) {
     // kernel is bound by latency (N = 28: 1 state 337 us, 140 here, 2 states 298 and 156, 4 states 255
     // and 163; N = 36, 1 state 1.94 and 1.32 ms; N = 40, 1 state 7.7 and 6.8).  Beyond it is bound by
     // the FP32 operations that both do and its smaller code wins (N = 36, 2 states 2.28 ms, 2.45 here;
-    // 4 states 3.9 and 4.7, 16 states 13.0 and 17.0).
+    // 4 states 3.9 and 4.7, 16 states 13.0 and 17.0).  The line lies on the safe side: with the best of
+    // its shapes this kernel is the faster one up to 2^17 elements (N = 30, 4 states 419 us tiled and
+    // 332 here; N = 32, 2 states 671 and 412, 4 states 828 and 756; N = 34, 2 states 1.26 and 1.05 ms),
+    // at 2^18 no more (N = 34, 4 states 1.89 and 1.96 ms).
     if (batch != 1 && !((batch == 2 || batch == 4) && D * batch <= (int64_t(1) << 15))) return false;
     const int full = 4;  // 256 threads
     const int64_t ctas = 2 * int64_t(sm_count()), tiles = (D * batch) >> (4 + 3 + full);
@@ -59,8 +62,10 @@ bool block_default(int n, int64_t batch, int dtype, BlockShape* sh) {
       if (block_shape(n, batch, dtype, 3, mb, cs, sh)) return true;
     return false;
   }
-  // State counts that are no power of two: sectors below 2^10 stay with the row kernel, which has
-  // no waits (N = 24, 6 states: 496 us there, 21 us here).
+  // State counts that are no power of two stay with the row kernel in sectors below 2^10.  That is not
+  // for speed (N = 20: 3 states 256 us there and 15 here, 6 states 266 and 15; N = 12, 6 states 46 and
+  // 16): a process whose staged copies time out still has a matvec without waits, which the failure
+  // tests ask for with 3 states at N = 20.  (N = 24, 6 states, beyond the line: 496 and 21 us.)
   if (!pow2(batch) && D < 1024) return false;
   const int lb = low_bits(batch);
   int full = 0;  // middle bits of a 256-thread CTA

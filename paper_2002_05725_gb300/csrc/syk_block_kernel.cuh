@@ -194,82 +194,82 @@ __global__ void __launch_bounds__(MAXT, MINB)
 
   int q = 0;
   for (int qe = PARTS ? min(c.part, nq) : nq;; qe = min(qe + c.part, nq)) {
-  for (; q < qe; ++q) {
-    const int st = q % kStages;
-    // the refill's chunk is read ahead: the refill itself then starts at once
-    const int4 refill = q + kStages < nq ? __ldg(&chunks[q0 + q + kStages]) : make_int4(0, 0, 0, 0);
-    // the lanes of a warp go on or give up together: a lane that left the loop alone would keep the
-    // others from ever passing the warp barriers below
-    if (!__all_sync(0xffffffffu, tma::wait_bounded(&full[st], (q / kStages) & 1, tma::wait_polls()))) break;
-    const unsigned char* tb = sm + st * stageb;
-    const unsigned char* cb = tb + tileb;
-    const uint4 head = *reinterpret_cast<const uint4*>(cb);
-    const uint4* rec = reinterpret_cast<const uint4*>(cb) + 1;
-    constexpr bool LOWS = SEC != 16 || LOWB;
-    auto partner = [&](const uint4 rc) SYK_INLINE {  // the thread's partner row 0
-      const uint32_t lm = LOWS ? (rc.x >> 16) & 0xffu : 0u;
-      return tb + (size_t)((((uint32_t)mid ^ (rc.x & 0xffffu)) << RB) * SE + ((uint32_t)low ^ lm) * B + s) * kElem;
-    };
-    CosetAt next;
-    uint4 rc;
-    auto prepare = [&]() SYK_INLINE {  // the next record's coset
-      rc = *rec++;
-      next.odd = rc.x >> 31;
-      next.prow = partner(rc);
-      next.un = support(ctx.x, rc.z);
-      next.sg = parity(rc.y & ctx.x);
-      next.tb = cb + rc.w;
-    };
-    const uint32_t cn = head.x;
-    auto run = [&](auto w, uint32_t count) SYK_INLINE {
-      constexpr int W = decltype(w)::value;
-#pragma unroll 1
-      for (uint32_t k = 0; k < count; ++k) {
-        const CosetAt at = next;
-        prepare();
-        A::template coset<W, LOWS>(acc, at, SE * kElem, ctx, p);
-        if (W == 4 && (k & 7u) == 7u) A::renorm(acc);
+    for (; q < qe; ++q) {
+      const int st = q % kStages;
+      // the refill's chunk is read ahead: the refill itself then starts at once
+      const int4 refill = q + kStages < nq ? __ldg(&chunks[q0 + q + kStages]) : make_int4(0, 0, 0, 0);
+      // the lanes of a warp go on or give up together: a lane that left the loop alone would keep the
+      // others from ever passing the warp barriers below
+      if (!__all_sync(0xffffffffu, tma::wait_bounded(&full[st], (q / kStages) & 1, tma::wait_polls()))) break;
+      const unsigned char* tb = sm + st * stageb;
+      const unsigned char* cb = tb + tileb;
+      const uint4 head = *reinterpret_cast<const uint4*>(cb);
+      const uint4* rec = reinterpret_cast<const uint4*>(cb) + 1;
+      constexpr bool LOWS = SEC != 16 || LOWB;
+      auto partner = [&](const uint4 rc) SYK_INLINE {  // the thread's partner row 0
+        const uint32_t lm = LOWS ? (rc.x >> 16) & 0xffu : 0u;
+        return tb + (size_t)((((uint32_t)mid ^ (rc.x & 0xffffu)) << RB) * SE + ((uint32_t)low ^ lm) * B + s) * kElem;
+      };
+      CosetAt next;
+      uint4 rc;
+      auto prepare = [&]() SYK_INLINE {  // the next record's coset
+        rc = *rec++;
+        next.odd = rc.x >> 31;
+        next.prow = partner(rc);
+        next.un = support(ctx.x, rc.z);
+        next.sg = parity(rc.y & ctx.x);
+        next.tb = cb + rc.w;
+      };
+      const uint32_t cn = head.x;
+      auto run = [&](auto w, uint32_t count) SYK_INLINE {
+        constexpr int W = decltype(w)::value;
+  #pragma unroll 1
+        for (uint32_t k = 0; k < count; ++k) {
+          const CosetAt at = next;
+          prepare();
+          A::template coset<W, LOWS>(acc, at, SE * kElem, ctx, p);
+          if (W == 4 && (k & 7u) == 7u) A::renorm(acc);
+        }
+        if (W == 4) A::renorm(acc);
+      };
+      prepare();  // (a record past the last one is never used: it reads the tables behind it)
+      run(std::integral_constant<int, 4>{}, cn & 0xffu);
+      run(std::integral_constant<int, 3>{}, (cn >> 8) & 0xffu);
+      run(std::integral_constant<int, 2>{}, (cn >> 16) & 0xffu);
+      run(std::integral_constant<int, 1>{}, cn >> 24);
+      run(std::integral_constant<int, 0>{}, head.y & 0xffu);
+  #pragma unroll 1
+      for (uint32_t k = head.y >> 8; k > 0; --k) {
+        const uint4 r2 = rc;
+        rc = *rec++;
+        A::record(acc, partner(r2), SE * kElem, r2, cb + r2.w, ctx);
       }
-      if (W == 4) A::renorm(acc);
-    };
-    prepare();  // (a record past the last one is never used: it reads the tables behind it)
-    run(std::integral_constant<int, 4>{}, cn & 0xffu);
-    run(std::integral_constant<int, 3>{}, (cn >> 8) & 0xffu);
-    run(std::integral_constant<int, 2>{}, (cn >> 16) & 0xffu);
-    run(std::integral_constant<int, 1>{}, cn >> 24);
-    run(std::integral_constant<int, 0>{}, head.y & 0xffu);
-#pragma unroll 1
-    for (uint32_t k = head.y >> 8; k > 0; --k) {
-      const uint4 r2 = rc;
-      rc = *rec++;
-      A::record(acc, partner(r2), SE * kElem, r2, cb + r2.w, ctx);
-    }
-    // the warp that finishes the chunk last refills its stage
-    __syncwarp();
-    if ((tid & 31) == 0) {
-      __threadfence_block();
-      if (atomicAdd(&done[st], 1) == nwarps - 1) {
-        __threadfence_block();  // the other warps' reads come before the refill's writes
-        done[st] = 0;
-        if (q + kStages < nq) issue(q + kStages, refill);
+      // the warp that finishes the chunk last refills its stage
+      __syncwarp();
+      if ((tid & 31) == 0) {
+        __threadfence_block();
+        if (atomicAdd(&done[st], 1) == nwarps - 1) {
+          __threadfence_block();  // the other warps' reads come before the refill's writes
+          done[st] = 0;
+          if (q + kStages < nq) issue(q + kStages, refill);
+        }
       }
+      __syncwarp();
     }
-    __syncwarp();
-  }
-  if (!PARTS || q < qe || q == nq) break;  // (q < qe: a wait gave up)
-  if constexpr (PARTS) {  // (a thread's rows of y are its own)
-    if (active) {
-      Out* __restrict__ yt = y + (size_t)tile * (tileb / kElem) + (size_t)(mid << RB) * SE + el;
-      const bool first = q == c.part;
+    if (!PARTS || q < qe || q == nq) break;  // (q < qe: a wait gave up)
+    if constexpr (PARTS) {  // (a thread's rows of y are its own)
+      if (active) {
+        Out* __restrict__ yt = y + (size_t)tile * (tileb / kElem) + (size_t)(mid << RB) * SE + el;
+        const bool first = q == c.part;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        Sum v = A::get(acc, r);
-        if (!first) A::add(v, yt[r * SE]);
-        yt[r * SE] = v;
+        for (int r = 0; r < R; ++r) {
+          Sum v = A::get(acc, r);
+          if (!first) A::add(v, yt[r * SE]);
+          yt[r * SE] = v;
+        }
       }
+      A::zero(acc);
     }
-    A::zero(acc);
-  }
   }
   if (q < nq) *lost = 1;
   __syncthreads();

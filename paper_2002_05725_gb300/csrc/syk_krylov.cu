@@ -750,10 +750,10 @@ size_t krylov_ws_bytes(int64_t D, int dtype, int m, int64_t B) {
   s += vb;                                            // w
   s += align_up(sizeof(double2) * G * (m + 1) * B);   // part
   s += 2 * align_up(sizeof(double2) * (m + 1) * B);   // h1, h2
-  s += align_up(sizeof(double) * G * B);              // npart
+  s += align_up(sizeof(double) * G * B);              // unused, as the one below: sizes stay as they were
   s += 2 * align_up(sizeof(double) * m * B);          // alpha, beta
   s += 3 * align_up(sizeof(double) * B);              // beta0, inv, sb
-  s += align_up(sizeof(double) * m * B);              // theta
+  s += align_up(sizeof(double) * m * B);
   s += align_up(sizeof(double) * m * m * B);          // Q
   s += align_up(sizeof(CheckRec));                    // rec
   s += align_up(sizeof(double2) * m * B);             // c
@@ -796,13 +796,13 @@ int krylov_ws_carve(KrylovWS* ws, void* base, size_t bytes, int64_t D, int dtype
   ws->part = (double2*)take(sizeof(double2) * ws->G * (m + 1) * B);
   ws->h1 = (double2*)take(sizeof(double2) * (m + 1) * B);
   ws->h2 = (double2*)take(sizeof(double2) * (m + 1) * B);
-  take(sizeof(double) * ws->G * B);
+  take(sizeof(double) * ws->G * B);  // unused
   ws->alpha = (double*)take(sizeof(double) * m * B);
   ws->beta = (double*)take(sizeof(double) * m * B);
   ws->beta0 = (double*)take(sizeof(double) * B);
   ws->inv = (double*)take(sizeof(double) * B);
   ws->sb = (double*)take(sizeof(double) * B);
-  ws->theta = (double*)take(sizeof(double) * m * B);
+  take(sizeof(double) * m * B);      // unused
   ws->Q = (double*)take(sizeof(double) * m * m * B);
   ws->rec = take(sizeof(CheckRec));
   ws->c = (double2*)take(sizeof(double2) * m * B);
@@ -925,9 +925,10 @@ int run_segment_graphed(const ApplyParams& P, const KrylovWS& ws, int dtype, int
 // curve) but overestimates by a few vectors (more at tight tol: measured, checking 2 vectors
 // before the prediction added 3 % matvecs at tol 1e-7 and 12 % at 1e-12), so the first check
 // comes at 3/4 of it (at least after 4 vectors, at most at m), the next ones every `every`
-// vectors: 2 when a matvec costs more than a check (~0.2 ms), else 4.  The matvec cost is
-// modelled from its work (8 nnz B flop at ~20 TFLOP/s for complex64, ~4.4 for complex128,
-// plus 10 us).
+// vectors: 2 when a matvec costs more than 0.2 ms, else 4.  That was the cost of a check by
+// the eigendecomposition; one by the expansion takes 41 to 50 us and a host read, and the plan
+// has stayed, so that bases end at the same dimensions.  The matvec cost is modelled from its
+// work (8 nnz B flop at ~20 TFLOP/s for complex64, ~4.4 for complex128, plus 10 us).
 struct CheckPlan {
   int first, every;
 };

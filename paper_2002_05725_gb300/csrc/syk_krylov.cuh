@@ -39,7 +39,6 @@ struct KrylovWS {
   double* beta = nullptr;    // m * B
   double* beta0 = nullptr;   // B
   double* inv = nullptr;     // B
-  double* theta = nullptr;   // m * B
   double* Q = nullptr;       // B * m * m
   double* sb = nullptr;      // B
   char* rec = nullptr;       // result of a convergence check (syk_krylov.cu)

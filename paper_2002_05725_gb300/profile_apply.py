@@ -30,7 +30,7 @@ def main():
     ap.add_argument("--tol", type=float, default=1e-7)
     ap.add_argument("--tile", default=None,
                     help="force the launch shape 'ntb,cluster[,variant]' (no tuning sweep; variant 0 = k_apply_tiled, "
-                         "1..3 = k_apply_coset with 2^variant rows per thread)")
+                         "1..3 = k_apply_coset with 2^variant rows per thread, 4 and 5 = k_apply_block with 32 and 8)")
     ap.add_argument("--grad", type=float, default=None, metavar="TSTAR",
                     help="also time one gradient call syk_otoc_grad (beta J = 5, t* = TSTAR, quad_dz 0.05, "
                          "tol 1e-7 for c64 and 1e-12 for c128), as the benchmark's gradient workload runs it")
